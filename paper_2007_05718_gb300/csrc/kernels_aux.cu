@@ -3,6 +3,7 @@
 // float32, frozen-cell overwrite and the FP64 energy-budget reductions.
 // Every population write also writes the site's periodic ghost mirrors.
 #include <algorithm>
+#include <cstring>
 #include <type_traits>
 
 #include "lb_rt_internal.h"
@@ -54,44 +55,6 @@ __global__ void k_init_state(Grid g, int Ni, int Next, const int* __restrict__ i
   }
 }
 
-// E, F, P per site: sums over directions in the table order.
-__global__ void k_moments(Grid g, int N, const void* __restrict__ pop, float* __restrict__ E,
-                          float* __restrict__ F, float* __restrict__ P, DirTable t) {
-  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (s >= g.sites) return;
-  int x, y, z;
-  site_xyz(g, s, x, y, z);
-  float e = 0, fx = 0, fy = 0, fz = 0, pxx = 0, pxy = 0, pxz = 0, pyy = 0, pyz = 0, pzz = 0;
-  for (int i = 0; i < N; ++i) {
-    const float v = load_pop(pop, g, i, z, y, x);
-    const float4 nw = t.nw[i];
-    e += v;
-    fx = fmaf(nw.x, v, fx);
-    fy = fmaf(nw.y, v, fy);
-    fz = fmaf(nw.z, v, fz);
-    pxx = fmaf(nw.x * nw.x, v, pxx);
-    pxy = fmaf(nw.x * nw.y, v, pxy);
-    pxz = fmaf(nw.x * nw.z, v, pxz);
-    pyy = fmaf(nw.y * nw.y, v, pyy);
-    pyz = fmaf(nw.y * nw.z, v, pyz);
-    pzz = fmaf(nw.z * nw.z, v, pzz);
-  }
-  if (E) E[s] = e;
-  if (F) {
-    F[s] = fx;
-    F[g.sites + s] = fy;
-    F[2 * g.sites + s] = fz;
-  }
-  if (P) {
-    P[s] = pxx;
-    P[g.sites + s] = pxy;
-    P[2 * g.sites + s] = pxz;
-    P[3 * g.sites + s] = pyy;
-    P[4 * g.sites + s] = pyz;
-    P[5 * g.sites + s] = pzz;
-  }
-}
-
 // Dense [Next][sites] float32 copy in the external direction order.
 __global__ void k_decode(Grid g, int Next, const int* __restrict__ int_of_ext,
                          const void* __restrict__ pop, float* __restrict__ out) {
@@ -106,22 +69,28 @@ __global__ void k_decode(Grid g, int Next, const int* __restrict__ int_of_ext,
 }
 
 // Frozen cells: overwrite, and add (prescribed - collided) energy to the
-// FP64 injection accumulator.
+// FP64 injection accumulator.  One warp per cell, lanes over the directions:
+// the cells are few, so what counts is the chain of dependent accesses (one
+// thread per cell walked its directions one after the other: 18.6 us for 32
+// cells x 16 directions).
 __global__ void k_frozen(Grid g, int Next, const int* __restrict__ int_of_ext, int ncells,
                          const int64_t* __restrict__ cells, const float* __restrict__ vals,
                          float* __restrict__ pop, double* injection) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (c >= ncells) return;
   int x, y, z;
   site_xyz(g, cells[c], x, y, z);
   double add = 0.0;
-  for (int e = 0; e < Next; ++e) {
+  for (int e = lane; e < Next; e += 32) {
     const int i = int_of_ext[e];
     const float v = vals[(size_t)c * Next + e];
-    add += (double)v - (double)pop[pidx(g, i, z, y, x)];
+    if (injection) add += (double)v - (double)pop[pidx(g, i, z, y, x)];
     store_pop(pop, g, i, z, y, x, v);
   }
-  if (injection) atomicAdd(injection, add);
+  if (injection) {
+    for (int s = 16; s > 0; s >>= 1) add += __shfl_xor_sync(0xffffffffu, add, s);
+    if (lane == 0) atomicAdd(injection, add);
+  }
 }
 
 // acc layout: [0] total, [1] initial, [2] outflow, [3] source, [4] injection,
@@ -272,43 +241,109 @@ __device__ __forceinline__ float f_at(const ST* pop, const float* e, const Grid&
   return fmaf(Eh, to_f<ST>(pop[pidx(g, i, z, y, x)]), Eh);
 }
 
-template <class ST>
-__global__ void k_moments16(Grid g, int N, const ST* __restrict__ pop, const float* __restrict__ e,
-                            float* __restrict__ E, float* __restrict__ F, float* __restrict__ P,
-                            DirTable t) {
-  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (s >= g.sites) return;
+// The site pair (x, x + 1), x even, of thread `p`: row base and coordinates.
+struct SitePair {
   int x, y, z;
-  site_xyz(g, s, x, y, z);
-  const float Eh = e[eidx(g, z, y, x)];
-  float es = 0, fx = 0, fy = 0, fz = 0, pxx = 0, pxy = 0, pxz = 0, pyy = 0, pyz = 0, pzz = 0;
-  for (int i = 0; i < N; ++i) {
-    const float4 nw = t.nw[i];
-    const float v = nw.w * fmaf(Eh, to_f<ST>(pop[pidx(g, i, z, y, x)]), Eh);
-    es += v;
+  bool in1;      // x + 1 inside
+  long long s;   // site of x
+};
+__device__ __forceinline__ bool site_pair(const Grid& g, long long p, SitePair& q) {
+  const unsigned npx = (unsigned)(g.nx + 1) / 2;  // sites < 2^31, so pairs and rows fit 32 bits
+  const unsigned r = (unsigned)p / npx;
+  if (p >= (long long)npx * g.ny * g.nz) return false;
+  q.x = 2 * (int)((unsigned)p - r * npx);
+  q.y = (int)(r % (unsigned)g.ny);
+  q.z = (int)(r / (unsigned)g.ny);
+  q.in1 = q.x + 1 < g.nx;
+  q.s = (long long)r * g.nx + q.x;
+  return true;
+}
+
+// populations (x, x + 1) of a direction row as float32 pair; 16-bit storage:
+// I = w E^ (1 + q)
+template <class ST>
+__device__ __forceinline__ float2 load_pair(const ST* p, float2 Eh, float w) {
+  if constexpr (std::is_same<ST, float>::value) {
+    return *reinterpret_cast<const float2*>(p);
+  } else {
+    const unsigned v = *reinterpret_cast<const unsigned*>(p);
+    ST lo, hi;
+    const unsigned short a = (unsigned short)v, b = (unsigned short)(v >> 16);
+    memcpy(&lo, &a, 2);
+    memcpy(&hi, &b, 2);
+    return make_float2(w * fmaf(Eh.x, to_f<ST>(lo), Eh.x), w * fmaf(Eh.y, to_f<ST>(hi), Eh.y));
+  }
+}
+
+// Moments of a site pair: sums over directions in the table order.  The rows
+// of padding and, past the end of an odd row, the ghost column are read and
+// not used.
+struct Moments {
+  float e = 0, fx = 0, fy = 0, fz = 0, pxx = 0, pxy = 0, pxz = 0, pyy = 0, pyz = 0, pzz = 0;
+  template <bool WITH_P>
+  __device__ __forceinline__ void add(float4 nw, float v) {
+    e += v;
     fx = fmaf(nw.x, v, fx);
     fy = fmaf(nw.y, v, fy);
     fz = fmaf(nw.z, v, fz);
-    pxx = fmaf(nw.x * nw.x, v, pxx);
-    pxy = fmaf(nw.x * nw.y, v, pxy);
-    pxz = fmaf(nw.x * nw.z, v, pxz);
-    pyy = fmaf(nw.y * nw.y, v, pyy);
-    pyz = fmaf(nw.y * nw.z, v, pyz);
-    pzz = fmaf(nw.z * nw.z, v, pzz);
+    if constexpr (WITH_P) {
+      pxx = fmaf(nw.x * nw.x, v, pxx);
+      pxy = fmaf(nw.x * nw.y, v, pxy);
+      pxz = fmaf(nw.x * nw.z, v, pxz);
+      pyy = fmaf(nw.y * nw.y, v, pyy);
+      pyz = fmaf(nw.y * nw.z, v, pyz);
+      pzz = fmaf(nw.z * nw.z, v, pzz);
+    }
   }
-  if (E) E[s] = es;
-  if (F) {
-    F[s] = fx;
-    F[g.sites + s] = fy;
-    F[2 * g.sites + s] = fz;
+};
+
+template <class ST, bool WITH_P>
+__device__ __forceinline__ void pair_moments(const Grid& g, int N, const ST* __restrict__ pop,
+                                             const float* __restrict__ e, const DirTable& t, const SitePair& q,
+                                             Moments& a, Moments& b) {
+  float2 Eh = make_float2(0.f, 0.f);
+  if constexpr (!std::is_same<ST, float>::value)
+    Eh = *reinterpret_cast<const float2*>(e + eidx(g, q.z, q.y, q.x));
+  const ST* p = pop + pidx(g, 0, q.z, q.y, q.x);
+#pragma unroll 4
+  for (int i = 0; i < N; ++i, p += g.si) {
+    const float4 nw = t.nw[i];
+    const float2 v = load_pair<ST>(p, Eh, nw.w);
+    a.add<WITH_P>(nw, v.x);
+    b.add<WITH_P>(nw, v.y);
   }
-  if (P) {
-    P[s] = pxx;
-    P[g.sites + s] = pxy;
-    P[2 * g.sites + s] = pxz;
-    P[3 * g.sites + s] = pyy;
-    P[4 * g.sites + s] = pyz;
-    P[5 * g.sites + s] = pzz;
+}
+
+// E, F, P of the current populations, two sites a thread: 8-byte (4-byte) loads
+// bring whole sectors, and E and F alone (no P) leave out six of ten sums.
+// 128^3 x 162 float16: 0.42 -> 0.14 ms (5.3 TB/s); 256^3 x 162 float32: 2.4 ->
+// 1.78 ms (6.7 TB/s), the rate of a plain copy.
+template <class ST, bool WITH_P>
+__global__ void k_moments(Grid g, int N, const ST* __restrict__ pop, const float* __restrict__ e,
+                          float* __restrict__ E, float* __restrict__ F, float* __restrict__ P,
+                          const __grid_constant__ DirTable t) {
+  SitePair q;
+  if (!site_pair(g, blockIdx.x * (long long)blockDim.x + threadIdx.x, q)) return;
+  Moments m[2];
+  pair_moments<ST, WITH_P>(g, N, pop, e, t, q, m[0], m[1]);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (k && !q.in1) return;
+    const long long s = q.s + k;
+    if (E) E[s] = m[k].e;
+    if (F) {
+      F[s] = m[k].fx;
+      F[g.sites + s] = m[k].fy;
+      F[2 * g.sites + s] = m[k].fz;
+    }
+    if (WITH_P && P) {
+      P[s] = m[k].pxx;
+      P[g.sites + s] = m[k].pxy;
+      P[2 * g.sites + s] = m[k].pxz;
+      P[3 * g.sites + s] = m[k].pyy;
+      P[4 * g.sites + s] = m[k].pyz;
+      P[5 * g.sites + s] = m[k].pzz;
+    }
   }
 }
 
@@ -334,26 +369,28 @@ __global__ void k_frozen16(Grid g, int Ni, int Next, const int* __restrict__ int
                            const int64_t* __restrict__ cells, const float* __restrict__ vals,
                            ST* __restrict__ pop, float* __restrict__ e, double* injection,
                            DirTable t) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (c >= ncells) return;
   int x, y, z;
   site_xyz(g, cells[c], x, y, z);
-  double old = 0.0, neu = 0.0;
-  for (int i = 0; i < Ni; ++i) old += (double)(t.nw[i].w * f_at(pop, e, g, i, z, y, x));
-  float E = 0.f;
-  for (int ex = 0; ex < Next; ++ex) {
-    E += vals[(size_t)c * Next + ex];
-    neu += (double)vals[(size_t)c * Next + ex];
-  }
+  float E = 0.f;  // every lane the whole sum, in the order of the directions
+#pragma unroll 8
+  for (int ex = 0; ex < Next; ++ex) E += vals[(size_t)c * Next + ex];
   const float Eh = fmaxf(E, EPS_E);
   const float ri = 1.f / Eh;
-  for (int ex = 0; ex < Next; ++ex) {
+  if (injection) {
+    double d = 0.0;  // prescribed - collided
+    for (int i = lane; i < Ni; i += 32) d -= (double)(t.nw[i].w * f_at(pop, e, g, i, z, y, x));
+    for (int ex = lane; ex < Next; ex += 32) d += (double)vals[(size_t)c * Next + ex];
+    for (int s = 16; s > 0; s >>= 1) d += __shfl_xor_sync(0xffffffffu, d, s);
+    if (lane == 0) atomicAdd(injection, d);
+  }
+  for (int ex = lane; ex < Next; ex += 32) {
     const int i = int_of_ext[ex];
     const float f = vals[(size_t)c * Next + ex] / t.nw[i].w;
     store_pop(pop, g, i, z, y, x, from_f<ST>(fmaf(f, ri, -1.f)));
   }
-  store_e_site(e, g, z, y, x, Eh);
-  if (injection) atomicAdd(injection, neu - old);
+  if (lane == 0) store_e_site(e, g, z, y, x, Eh);
 }
 
 template <class ST>
@@ -390,70 +427,59 @@ __global__ void k_total_partials16(Grid g, int N, const ST* __restrict__ pop,
 // form against the E array `e`.
 template <class ST>
 __global__ void k_coupling(Grid g, int N, const ST* __restrict__ pop, const float* __restrict__ e,
-                           DirTable t, MovingCoef c, float* __restrict__ Jo, float* __restrict__ Ho,
-                           float* __restrict__ So) {
-  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (s >= g.sites) return;
-  int x, y, z;
-  site_xyz(g, s, x, y, z);
-  float Eh = 0.f;
-  if (!std::is_same<ST, float>::value) Eh = e[eidx(g, z, y, x)];
-  float E = 0, Fx = 0, Fy = 0, Fz = 0, Pxx = 0, Pxy = 0, Pxz = 0, Pyy = 0, Pyz = 0, Pzz = 0;
-  for (int i = 0; i < N; ++i) {
-    const float4 nw = t.nw[i];
-    float I;
-    if constexpr (std::is_same<ST, float>::value) I = pop[pidx(g, i, z, y, x)];
-    else I = nw.w * fmaf(Eh, to_f<ST>(pop[pidx(g, i, z, y, x)]), Eh);
-    E += I;
-    Fx = fmaf(nw.x, I, Fx);
-    Fy = fmaf(nw.y, I, Fy);
-    Fz = fmaf(nw.z, I, Fz);
-    Pxx = fmaf(nw.x * nw.x, I, Pxx);
-    Pxy = fmaf(nw.x * nw.y, I, Pxy);
-    Pxz = fmaf(nw.x * nw.z, I, Pxz);
-    Pyy = fmaf(nw.y * nw.y, I, Pyy);
-    Pyz = fmaf(nw.y * nw.z, I, Pyz);
-    Pzz = fmaf(nw.z * nw.z, I, Pzz);
-  }
-  const float vx = c.v ? c.v[s] : 0.f, vy = c.v ? c.v[g.sites + s] : 0.f,
-              vz = c.v ? c.v[2 * g.sites + s] : 0.f;
-  const float W2 = 1.f / (1.f - (vx * vx + vy * vy + vz * vz));
-  const float W = sqrtf(W2);
-  const float Fv = Fx * vx + Fy * vy + Fz * vz;
-  // Pv_i = P^ik v_k
-  const float Pvx = Pxx * vx + Pxy * vy + Pxz * vz;
-  const float Pvy = Pxy * vx + Pyy * vy + Pyz * vz;
-  const float Pvz = Pxz * vx + Pyz * vy + Pzz * vz;
-  const float Pvv = Pvx * vx + Pvy * vy + Pvz * vz;
-  const float J = W2 * (E - 2.f * Fv + Pvv);
-  // h_ji a^i = a_j + W^2 v_j (v.a) for a = F - Pv
-  const float ax = Fx - Pvx, ay = Fy - Pvy, az = Fz - Pvz;
-  const float va = vx * ax + vy * ay + vz * az;
-  const float c1 = W * W2 * (Fv - E), c2 = W * W2 * va;
-  const float Hx = c1 * vx + W * ax + c2 * vx;
-  const float Hy = c1 * vy + W * ay + c2 * vy;
-  const float Hz = c1 * vz + W * az + c2 * vz;
-  if (Jo) Jo[s] = J;
-  if (Ho) {
-    Ho[s] = Hx;
-    Ho[g.sites + s] = Hy;
-    Ho[2 * g.sites + s] = Hz;
-  }
-  if (So) {
-    const float kta = c.kta ? c.kta[s] : c.kta_s, kt0 = c.kt0 ? c.kt0[s] : c.kt0_s;
-    const float etat = c.etat ? c.etat[s] : c.etat_s;
-    const float kt = kta + kt0;
-    // time component of the comoving flux four-vector, H^mu u_mu = 0
-    const float H0 = vx * Hx + vy * Hy + vz * Hz;
-    const float emit = W * (kta * J - etat);
-    So[s] = fmaf(kt, H0, emit);
-    So[g.sites + s] = fmaf(kt, Hx, emit * vx);
-    So[2 * g.sites + s] = fmaf(kt, Hy, emit * vy);
-    So[3 * g.sites + s] = fmaf(kt, Hz, emit * vz);
+                           const __grid_constant__ DirTable t, MovingCoef c, float* __restrict__ Jo,
+                           float* __restrict__ Ho, float* __restrict__ So) {
+  SitePair q;
+  if (!site_pair(g, blockIdx.x * (long long)blockDim.x + threadIdx.x, q)) return;
+  Moments mm[2];
+  pair_moments<ST, true>(g, N, pop, e, t, q, mm[0], mm[1]);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (k && !q.in1) return;
+    const long long s = q.s + k;
+    const float E = mm[k].e, Fx = mm[k].fx, Fy = mm[k].fy, Fz = mm[k].fz, Pxx = mm[k].pxx, Pxy = mm[k].pxy,
+                Pxz = mm[k].pxz, Pyy = mm[k].pyy, Pyz = mm[k].pyz, Pzz = mm[k].pzz;
+    const float vx = c.v ? c.v[s] : 0.f, vy = c.v ? c.v[g.sites + s] : 0.f,
+                vz = c.v ? c.v[2 * g.sites + s] : 0.f;
+    const float W2 = 1.f / (1.f - (vx * vx + vy * vy + vz * vz));
+    const float W = sqrtf(W2);
+    const float Fv = Fx * vx + Fy * vy + Fz * vz;
+    // Pv_i = P^ik v_k
+    const float Pvx = Pxx * vx + Pxy * vy + Pxz * vz;
+    const float Pvy = Pxy * vx + Pyy * vy + Pyz * vz;
+    const float Pvz = Pxz * vx + Pyz * vy + Pzz * vz;
+    const float Pvv = Pvx * vx + Pvy * vy + Pvz * vz;
+    const float J = W2 * (E - 2.f * Fv + Pvv);
+    // h_ji a^i = a_j + W^2 v_j (v.a) for a = F - Pv
+    const float ax = Fx - Pvx, ay = Fy - Pvy, az = Fz - Pvz;
+    const float va = vx * ax + vy * ay + vz * az;
+    const float c1 = W * W2 * (Fv - E), c2 = W * W2 * va;
+    const float Hx = c1 * vx + W * ax + c2 * vx;
+    const float Hy = c1 * vy + W * ay + c2 * vy;
+    const float Hz = c1 * vz + W * az + c2 * vz;
+    if (Jo) Jo[s] = J;
+    if (Ho) {
+      Ho[s] = Hx;
+      Ho[g.sites + s] = Hy;
+      Ho[2 * g.sites + s] = Hz;
+    }
+    if (So) {
+      const float kta = c.kta ? c.kta[s] : c.kta_s, kt0 = c.kt0 ? c.kt0[s] : c.kt0_s;
+      const float etat = c.etat ? c.etat[s] : c.etat_s;
+      const float kt = kta + kt0;
+      // time component of the comoving flux four-vector, H^mu u_mu = 0
+      const float H0 = vx * Hx + vy * Hy + vz * Hz;
+      const float emit = W * (kta * J - etat);
+      So[s] = fmaf(kt, H0, emit);
+      So[g.sites + s] = fmaf(kt, Hx, emit * vx);
+      So[2 * g.sites + s] = fmaf(kt, Hy, emit * vy);
+      So[3 * g.sites + s] = fmaf(kt, Hz, emit * vz);
+    }
   }
 }
 
 unsigned grid1d(long long n) { return (unsigned)((n + BLK - 1) / BLK); }
+unsigned pair_grid(const Grid& g) { return grid1d((long long)((g.nx + 1) / 2) * g.ny * g.nz); }
 
 }  // namespace
 
@@ -474,14 +500,15 @@ cudaError_t launch_init_state(const Grid& g, int Ni, int Next, const int* int_of
 
 cudaError_t launch_moments(const Grid& g, int N, const void* pop, const float* e, int storage,
                            const DirTable& t, float* E, float* F, float* P, cudaStream_t s) {
-  if (storage == ST_F32)
-    k_moments<<<grid1d(g.sites), BLK, 0, s>>>(g, N, pop, E, F, P, t);
-  else if (storage == ST_F16)
-    k_moments16<__half><<<grid1d(g.sites), BLK, 0, s>>>(g, N, static_cast<const __half*>(pop), e,
-                                                        E, F, P, t);
-  else
-    k_moments16<__nv_bfloat16><<<grid1d(g.sites), BLK, 0, s>>>(
-        g, N, static_cast<const __nv_bfloat16*>(pop), e, E, F, P, t);
+  auto go = [&](auto tag) {
+    using ST = decltype(tag);
+    const ST* p = static_cast<const ST*>(pop);
+    if (P) k_moments<ST, true><<<pair_grid(g), BLK, 0, s>>>(g, N, p, e, E, F, P, t);
+    else k_moments<ST, false><<<pair_grid(g), BLK, 0, s>>>(g, N, p, e, E, F, P, t);
+  };
+  if (storage == ST_F32) go(float());
+  else if (storage == ST_F16) go(__half());
+  else go(__nv_bfloat16());
   return cudaGetLastError();
 }
 
@@ -503,7 +530,7 @@ cudaError_t launch_frozen(const Grid& g, int Ni, int Next, const int* int_of_ext
                           const int64_t* cells, const float* vals, void* pop, float* e,
                           int storage, const DirTable& t, double* injection_acc, cudaStream_t s) {
   if (ncells <= 0) return cudaSuccess;
-  const int nb = (ncells + BLK - 1) / BLK;
+  const int nb = (ncells + BLK / 32 - 1) / (BLK / 32);  // a warp per cell
   if (storage == ST_F32)
     k_frozen<<<nb, BLK, 0, s>>>(g, Next, int_of_ext, ncells, cells, vals,
                                 static_cast<float*>(pop), injection_acc);
@@ -521,13 +548,13 @@ cudaError_t launch_coupling(const Grid& g, int N, const void* pop, const float* 
                             const DirTable& t, const MovingCoef& c, float* J, float* H, float* S,
                             cudaStream_t s) {
   if (storage == ST_F32)
-    k_coupling<float><<<grid1d(g.sites), BLK, 0, s>>>(g, N, static_cast<const float*>(pop), e, t,
+    k_coupling<float><<<pair_grid(g), BLK, 0, s>>>(g, N, static_cast<const float*>(pop), e, t,
                                                       c, J, H, S);
   else if (storage == ST_F16)
-    k_coupling<__half><<<grid1d(g.sites), BLK, 0, s>>>(g, N, static_cast<const __half*>(pop), e,
+    k_coupling<__half><<<pair_grid(g), BLK, 0, s>>>(g, N, static_cast<const __half*>(pop), e,
                                                        t, c, J, H, S);
   else
-    k_coupling<__nv_bfloat16><<<grid1d(g.sites), BLK, 0, s>>>(
+    k_coupling<__nv_bfloat16><<<pair_grid(g), BLK, 0, s>>>(
         g, N, static_cast<const __nv_bfloat16*>(pop), e, t, c, J, H, S);
   return cudaGetLastError();
 }
