@@ -13,6 +13,7 @@
 
 #include "handle.h"
 #include "lb_rt_internal.h"
+#include "static_step.h"
 
 using namespace lbrt;
 
@@ -82,7 +83,7 @@ struct lb_rt_batch {
   CUtensorMap* h_maps = nullptr;
   CUtensorMap* d_maps = nullptr;
   bool maps_dirty = true;
-  unsigned* d_err = nullptr;
+  unsigned* d_err = nullptr;  // error word, then the tile counters (4 words)
   // one graph per tick parity; the launch plan it was captured for: per
   // launch (group, first descriptor, problems, tiles) and per descriptor
   // (slot, z chunks); a graph is replayed only for an identical plan, and a
@@ -150,9 +151,9 @@ bool same_table(const Group& g, const lb_rt* h) {
 // second group's (b_*) in the same launch, its problems on CTAs ctas_a ..
 // ctas - 1.
 struct Launch {
-  int group, first, nprob, ntiles, periodic;
+  int group, first, nprob, ntiles, flux;
   long long sd = 0;  // site-direction updates of the launch's problems of `group`
-  int b_group = -1, b_first = 0, b_nprob = 0, b_ntiles = 0, b_periodic = 0;
+  int b_group = -1, b_first = 0, b_nprob = 0, b_ntiles = 0, b_flux = 0;
   long long b_sd = 0;
   int ctas_a = 0, ctas = 0;
 };
@@ -193,12 +194,12 @@ lb_rt_status lb_rt_batch_create(const lb_rt_batch_config* cfg, lb_rt_batch** out
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_maps, sizeof(CUtensorMap) * nmaps);
   if (e == cudaSuccess) std::memset(b->h_maps, 0, sizeof(CUtensorMap) * nmaps);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_maps, sizeof(CUtensorMap) * nmaps);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_err, sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_err, 5 * sizeof(unsigned));
   for (int i = 0; i < lb_rt_batch::kTickEvents && e == cudaSuccess; ++i)
     e = cudaEventCreateWithFlags(&b->tick_ev[i], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreate(&b->pev0);
   if (e == cudaSuccess) e = cudaEventCreate(&b->pev1);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, sizeof(unsigned), b->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, 5 * sizeof(unsigned), b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
     lb_rt_batch_destroy(b);
@@ -295,7 +296,7 @@ lb_rt_status lb_rt_batch_admit(lb_rt_batch* b, const lb_rt_config* cfg, const lb
     g.Ni = h->Ni;
     g.dpt = h->dpt;
     g.zc = h->zc;
-    cudaError_t e = occupancy_static_batch(c.storage, g.dpt, g.zc, g.Ni / g.dpt, &g.per_sm);
+    cudaError_t e = occupancy_static_batch(c.storage, g.dpt, g.zc, g.Ni, &g.per_sm);
     if (e == cudaSuccess && g.per_sm < 1) e = cudaErrorInvalidConfiguration;
     if (e == cudaSuccess) e = cudaEventCreate(&g.ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&g.ev1);
@@ -306,10 +307,9 @@ lb_rt_status lb_rt_batch_admit(lb_rt_batch* b, const lb_rt_config* cfg, const lb
     }
     for (int z : kZCandidates) g.cands.push_back(z);
     g.cost.assign(g.cands.size() + 1, 0.0);  // z chunks, then the alternative kernel
-    g.alt_zc = batch_alt_zc(c.storage, g.dpt);
+    g.alt_zc = batch_alt_zc(g.dpt, g.zc);
     if (g.alt_zc &&
-        (occupancy_static_batch(c.storage, g.dpt, g.alt_zc, g.Ni / g.dpt, &g.alt_per_sm, 1) !=
-             cudaSuccess ||
+        (occupancy_static_batch(c.storage, g.dpt, g.zc, g.Ni, &g.alt_per_sm, 1) != cudaSuccess ||
          g.alt_per_sm < 1)) {
       (void)cudaGetLastError();
       g.alt_zc = 0;
@@ -389,6 +389,9 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
   std::vector<std::vector<std::vector<int>>> plan(K, std::vector<std::vector<int>>(G));
   int active = 0;
   std::vector<long long> group_sd(G, 0);
+  // groups with flux terms (lambda != 0): where those take other boxes than
+  // the plan's own kernel, the maps are the alternative kernel's
+  std::vector<int> group_flux(G, 0), group_maps(G, 0);
   for (int s = 0; s < (int)b->slots.size(); ++s) {
     const Member& m = b->slots[s];
     if (!m.used) continue;
@@ -398,6 +401,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     const long long take = std::min<long long>(rem, K);
     for (int k = 0; k < take; ++k) plan[k][m.group].push_back(s);
     group_sd[m.group] += take * m.h->grid.sites;
+    if (has_flux(m.h->sc)) group_flux[m.group] = 1;
   }
   if (n_active) *n_active = active;
   if (!active) return LB_RT_OK;
@@ -436,11 +440,10 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     if (act.size() == 2) {
       const Group& g0 = b->groups[act[0]];
       const Group& g1 = b->groups[act[1]];
-      const int st = b->cfg.storage;
-      if (static_batch_pair_supported(st, g0.dpt, g0.zc_now(), g1.dpt, g1.zc_now())) {
+      if (static_batch_pair_supported(g0.dpt, g0.zc_now(), g1.dpt, g1.zc_now())) {
         pa = act[0];
         pb = act[1];
-      } else if (static_batch_pair_supported(st, g1.dpt, g1.zc_now(), g0.dpt, g0.zc_now())) {
+      } else if (static_batch_pair_supported(g1.dpt, g1.zc_now(), g0.dpt, g0.zc_now())) {
         pa = act[1];
         pb = act[0];
       }
@@ -450,8 +453,8 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     const Group& A = b->groups[pa];
     const Group& B = b->groups[pb];
     int per_sm = 0;
-    cudaError_t e = occupancy_static_batch_pair(b->cfg.storage, A.dpt, A.zc_now(), A.Ni / A.dpt,
-                                                B.dpt, B.zc_now(), B.Ni / B.dpt, &per_sm);
+    cudaError_t e = occupancy_static_batch_pair(b->cfg.storage, A.dpt, A.zc_now(), A.Ni, B.dpt,
+                                                B.zc_now(), B.Ni, &per_sm);
     if (e != cudaSuccess) return bcuda(b, e, "paired kernel occupancy");
     b->pair_a = pa;
     b->pair_b = pb;
@@ -476,6 +479,16 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       if (b->pair_trial == 0) pa = pb = -1;  // first trial: separate launches
     } else if (b->pair_choice == 0) {
       pa = pb = -1;
+    }
+  }
+  if (pa >= 0 && (group_flux[pa] || group_flux[pb])) group_flux[pa] = group_flux[pb] = 1;  // one kernel
+  for (int g = 0; g < G; ++g) {
+    const Group& gr = b->groups[g];
+    group_maps[g] = gr.alt;
+    if (group_flux[g] && gr.zc != static_flux_zc(gr.dpt)) {
+      if (gr.alt_zc != static_flux_zc(gr.dpt))
+        return bfail(b, LB_RT_ECUDA, "no tensor maps for the flux terms of this tile plan");
+      group_maps[g] = 1;
     }
   }
   // descriptor tables [step][group members]
@@ -519,19 +532,20 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
         d.g = h->grid;
         d.out = h->pop[cur ^ 1];
         d.e_out = h->ef[cur ^ 1];
-        d.tmap = b->d_maps + (size_t)s * 8 + gr.alt * 4 + cur * 2;
-        d.emap = b->d_maps + (size_t)s * 8 + gr.alt * 4 + cur * 2 + 1;
+        d.tmap = b->d_maps + (size_t)s * 8 + group_maps[g] * 4 + cur * 2;
+        d.emap = b->d_maps + (size_t)s * 8 + group_maps[g] * 4 + cur * 2 + 1;
         d.cf = h->sc;
         d.dt = (float)h->dt;
         d.collision = h->cfg.collision;
         d.lambda_iters = h->cfg.lambda_iters;
-        d.nzc = std::max(1, std::min(h->grid.nz, (h->grid.nz + gr.zchunk - 1) / gr.zchunk));
+        const int march = march_length(h->grid);
+        d.nzc = std::max(1, std::min(march, (march + gr.zchunk - 1) / gr.zchunk));
         d.tile_start = L.ntiles;
-        d.ntiles = (h->grid.nx + 63) / 64 * h->grid.ny * d.nzc;
+        d.ntiles = static_tiles(h->grid, d.nzc);
         d.budget_partials = nullptr;
         L.ntiles += d.ntiles;
         L.sd += h->grid.sites * (long long)gr.Ni;
-        if (h->grid.periodic[0] || h->grid.periodic[1] || h->grid.periodic[2]) L.periodic = 1;
+        L.flux = group_flux[g];
         sig.push_back(s);
         sig.push_back(d.nzc);
       }
@@ -558,7 +572,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
         A.b_first = Bl.first;
         A.b_nprob = Bl.nprob;
         A.b_ntiles = Bl.ntiles;
-        A.b_periodic = Bl.periodic;
+        A.b_flux = Bl.flux;
         A.b_sd = Bl.sd;
         A.ctas_a = (int)ca;
         A.ctas = (int)S;
@@ -568,9 +582,9 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     }
     for (size_t i = first_of_step; i < launches.size(); ++i) {
       const Launch& L = launches[i];
-      for (long long v : {(long long)L.group, (long long)b->groups[L.group].alt,
+      for (long long v : {(long long)L.group, (long long)group_maps[L.group],
                           (long long)L.first, (long long)L.nprob,
-                          (long long)L.ntiles, (long long)L.periodic, (long long)L.b_group,
+                          (long long)L.ntiles, (long long)L.flux, (long long)L.b_group,
                           (long long)L.b_first, (long long)L.b_nprob, (long long)L.b_ntiles,
                           (long long)L.ctas_a, (long long)L.ctas})
         sig.push_back(v);
@@ -594,7 +608,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(d_desc, h_desc, sizeof(ProblemDesc) * ndesc, cudaMemcpyHostToDevice,
                           b->stream);
-    auto batch_of = [&](int g, int first, int nprob, int ntiles, int periodic, int ctas) {
+    auto batch_of = [&](int g, int first, int nprob, int ntiles, int flux, int ctas) {
       const Group& gr = b->groups[g];
       BatchLaunch B{};
       B.table = d_desc + first;
@@ -606,8 +620,9 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       B.alt = gr.alt;
       B.storage = b->cfg.storage;
       B.ctas = ctas;
-      B.periodic = periodic;
+      B.flux = flux;
       B.err = b->d_err;
+      B.sched = b->d_err + 1;
       return B;
     };
     auto single = [&](const Launch& L) -> cudaError_t {
@@ -617,7 +632,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       gr.last_zc = gr.zc_now();
       gr.ctas = ctas;
       gr.paired = false;
-      return launch_tma_static_batch(batch_of(L.group, L.first, L.nprob, L.ntiles, L.periodic, ctas),
+      return launch_static_batch(batch_of(L.group, L.first, L.nprob, L.ntiles, L.flux, ctas),
                                      gr.table, b->stream);
     };
     if (timed && tuning) {
@@ -640,9 +655,9 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       }
       Group& ga = b->groups[L.group];
       Group& gb = b->groups[L.b_group];
-      const BatchLaunch A = batch_of(L.group, L.first, L.nprob, L.ntiles, L.periodic, L.ctas_a);
+      const BatchLaunch A = batch_of(L.group, L.first, L.nprob, L.ntiles, L.flux, L.ctas_a);
       const BatchLaunch B =
-          batch_of(L.b_group, L.b_first, L.b_nprob, L.b_ntiles, L.b_periodic, L.ctas - L.ctas_a);
+          batch_of(L.b_group, L.b_first, L.b_nprob, L.b_ntiles, L.b_flux, L.ctas - L.ctas_a);
       ga.ctas = L.ctas_a;
       gb.ctas = L.ctas - L.ctas_a;
       ga.last_zc = ga.zc_now();

@@ -17,8 +17,8 @@ struct lb_rt {
   int N = 0;                    // directions, external (user) order
   int Ni = 0;                   // internal directions including inert padding
   int dpt = 0, zc = 0;          // tile plan of the static kernel
-  bool pipelined = false;       // single-problem static steps run the pipelined kernel
   int nzc = 0, ctas = 0;        // its persistent grid: z chunks, CTAs
+  int nzc_flux = 0, ctas_flux = 0;  // the same for the flux terms
   std::vector<int> ext_of_int;  // internal -> external index (-1: padding)
   std::vector<int> int_of_ext;  // external -> internal index
   int* d_int_of_ext = nullptr;  // device copy
@@ -32,6 +32,7 @@ struct lb_rt {
   float* ef[2] = {nullptr, nullptr};   // 16-bit storage: padded E arrays paired with pop[]
   size_t ef_bytes = 0;
   CUtensorMap tmap[2];                 // TMA descriptors of pop[0] / pop[1]
+  CUtensorMap tmap_flux[2], emap_flux[2];  // the same with static_flux_zc planes (where that differs)
   CUtensorMap emap[2];                 // 16-bit storage: TMA descriptors of ef[0] / ef[1]
   bool tmap_ok = false;
   bool iso = false;             // isotropic table: sum w = 1, sum w n = 0, sum w n n = Id / d
@@ -47,7 +48,7 @@ struct lb_rt {
   double* partials = nullptr;
   int partials_cap = 0;
   double* acc = nullptr;       // 8 doubles, see k_budget_finalize
-  unsigned* err = nullptr;     // device error word
+  unsigned* err = nullptr;     // device error word, followed by the 2 words of the tile counter
   unsigned* err_host = nullptr;  // page-locked host copy of it, read after each sync
   float* scratch = nullptr;    // moments staging for host outputs [10][sites]
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;

@@ -3,7 +3,7 @@
 // al. 2020, App. B, with the streaming of Sec. 3.3 (Eq. interp).
 //
 // Tiles, boxes, the TMA ring and the z-sweep with the carried plane are those
-// of the static kernel (kernels_tma.cu), one plane per batch.  The collision
+// of the static kernel (kernels_static.cuh), one plane per batch.  The collision
 // is per site and direction: with W = (1 - v^2)^(-1/2), beta_i = 1 - v.n_i,
 //   A_i = 1 / (1 + dt W beta_i (kt_a + kt_0)),  g_i = A_i dt w_i (W beta_i)^-3,
 //   I_i^{n+1} = A_i I*_i + g_i (eta_t + kt_0 J),

@@ -105,69 +105,47 @@ void plan_directions(lb_rt* h) {
       std::stable_sort(c.begin(), c.end(), [&](int a, int b) {
         return (h->n[3 * a] < 0) < (h->n[3 * b] < 0);
       });
-    // the first plan (in the kernel's order of preference) that fits and
-    // pads the direction set by at most 4 % more than the tightest plan
-    // (a moving fluid with no fitting plan falls back to the one-thread-per-
-    // site kernel with this ordering and no padding).  A static handle
-    // prefers the pipelined kernel's plans; the plan it takes must also fit
-    // the first-generation kernel, which runs the batched launches (the
-    // direction grouping fixes the summation order, so a problem gives the
-    // same bits on both).
-    const bool f32 = h->cfg.storage == LB_RT_F32;
-    const bool mov = h->cfg.moving != 0;
-    const int (*old_plans)[3] = mov ? kTilePlansMoving : f32 ? kTilePlans : kTilePlans16;
-    const int n_old = mov ? kNumTilePlansMoving : f32 ? kNumTilePlans : kNumTilePlans16;
+    // the first plan (in order of preference) that fits and pads the
+    // direction set by at most 4 % more than the tightest plan of its list (a
+    // moving fluid with no fitting plan falls back to the one-thread-per-site
+    // kernel with this ordering and no padding)
     auto pad_ni = [&](int dpt) {
       int ni = 0;
       for (auto& c : cls) ni += (int)(c.size() + dpt - 1) / dpt * dpt;
       return ni;
     };
-    auto old_fits = [&](int dpt, int zc) {
-      for (int p = 0; p < n_old; ++p) {
-        if (old_plans[p][0] != dpt || old_plans[p][1] != zc) continue;
-        if (zc > 1 && zc > h->grid.nz) return false;
-        const int ni = pad_ni(dpt), warps = ni / dpt;
-        if (ni > kMaxInternalDirs || 32 * warps > old_plans[p][2]) return false;
-        const size_t smem = mov ? step_tile_smem_moving(dpt, warps)
-                            : f32 ? step_tile_smem(dpt, zc, warps) : step_tile_smem16(dpt, zc, warps);
-        return smem <= 226 * 1024;
-      }
-      return false;
-    };
-    auto choose = [&](const int (*plans)[3], int nplans, bool sc) {
+    auto choose = [&](int nplans, auto dpt_of, auto fits) {
       std::vector<int> ni_of(nplans, -1);
       int min_ni = 1 << 30;
       for (int p = 0; p < nplans; ++p) {
-        const int dpt = plans[p][0], zc = plans[p][1];
-        if (!old_fits(dpt, zc)) continue;
-        const int ni = pad_ni(dpt), warps = ni / dpt;
-        if (sc && (32 * (warps + zc) > plans[p][2] ||
-                   step_tile_smem_sc(h->cfg.storage, dpt, zc, warps) > 226 * 1024))
-          continue;
+        const int ni = pad_ni(dpt_of(p));
+        if (ni > kMaxInternalDirs || !fits(p, ni / dpt_of(p))) continue;
         ni_of[p] = ni;
         min_ni = std::min(min_ni, ni);
       }
       for (int p = 0; p < nplans; ++p)
-        if (ni_of[p] >= 0 && ni_of[p] * 100 <= min_ni * 104) return p;
-      return -1;
+        if (ni_of[p] >= 0 && ni_of[p] * 100 <= min_ni * 104) return dpt_of(p);
+      return 0;
     };
-    int best = -1;
-    h->pipelined = false;
-    // float32 populations keep the first-generation kernel, which measured
-    // faster on the 42- and 162-direction workloads; 16-bit storage takes the
-    // pipelined one
-    if (!mov && !f32) {
-      best = choose(kTilePlansSC, kNumTilePlansSC, true);
-      if (best >= 0) {
-        h->pipelined = true;
-        h->dpt = kTilePlansSC[best][0];
-        h->zc = kTilePlansSC[best][1];
-      }
-    }
-    if (best < 0) {
-      best = choose(old_plans, n_old, false);
-      h->dpt = best >= 0 ? old_plans[best][0] : 0;
-      h->zc = best >= 0 ? old_plans[best][1] : 0;
+    h->dpt = 0;
+    if (h->cfg.moving) {
+      h->dpt = choose(kNumTilePlansMoving, [](int p) { return kTilePlansMoving[p][0]; },
+                      [&](int p, int warps) {
+                        return 32 * warps <= kTilePlansMoving[p][2] &&
+                               step_tile_smem_moving(kTilePlansMoving[p][0], warps) <= 226 * 1024;
+                      });
+      h->zc = h->dpt ? 1 : 0;
+    } else {
+      const TilePlan* lists[2] = {nullptr, nullptr};
+      int counts[2] = {0, 0};
+      const int nlists = static_plan_lists(h->cfg.storage, lists, counts);
+      for (int l = 0; l < nlists && !h->dpt; ++l)
+        h->dpt = choose(counts[l], [&](int p) { return lists[l][p].dpt; },
+                        [&](int p, int warps) {
+                          const TilePlan& t = lists[l][p];
+                          return (t.planes == 1 || t.planes <= h->grid.nz) && warps <= t.max_warps;
+                        });
+      h->zc = h->dpt ? static_zc(h->dpt, h->grid) : 0;
     }
     for (auto& c : cls) {
       for (int e : c) h->ext_of_int.push_back(e);
@@ -251,11 +229,17 @@ lb_rt_status run_steps(lb_rt* h, int nsteps, float* mE, float* mF) {
     L.in = h->pop[h->cur];
     L.out = h->pop[h->cur ^ 1];
     L.tmap_in = h->tmap_ok ? &h->tmap[h->cur] : nullptr;
+    if (!h->cfg.moving && h->zc != static_flux_zc(h->dpt)) {
+      L.tmap_flux = &h->tmap_flux[h->cur];
+      L.tmap_e_flux = h->ef[0] ? &h->emap_flux[h->cur] : nullptr;
+      L.nzc_flux = h->nzc_flux;
+      L.ctas_flux = h->ctas_flux;
+    }
     L.tmap_e = h->ef[0] && h->tmap_ok ? &h->emap[h->cur] : nullptr;
     L.e_in = h->ef[h->cur];
     L.e_out = h->ef[h->cur ^ 1];
     L.err = h->err;
-    L.sc = h->pipelined;
+    L.sched = h->err + 1;
     L.budget_partials = nullptr;
     L.partials_cap = h->partials_cap;
     if (s == nsteps - 1) {
@@ -313,6 +297,7 @@ size_t lbrt::handle_device_bytes(const lb_rt_config& cfg, std::string& err) {
   tmp.grid.nx = cfg.nx;
   tmp.grid.ny = cfg.ny;
   tmp.grid.nz = cfg.nz;
+  tmp.grid.dims = cfg.dims;
   plan_directions(&tmp);
   if (!cfg.moving && !tmp.dpt) {
     err = "no tile plan fits this direction set";
@@ -434,7 +419,7 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
   alloc((void**)&h->partials, sizeof(double) * 2 * h->partials_cap);
   alloc((void**)&h->acc, sizeof(double) * 8);
   alloc((void**)&h->d_int_of_ext, sizeof(int) * h->N);
-  alloc((void**)&h->err, sizeof(unsigned));
+  alloc((void**)&h->err, 3 * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->err_host, sizeof(unsigned), cudaHostAllocDefault);
   if (e != cudaSuccess) {
     g_create_msg = std::string("allocation: ") + cudaGetErrorString(e);
@@ -452,7 +437,7 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->d_int_of_ext, h->int_of_ext.data(), sizeof(int) * h->N,
                         cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, 3 * sizeof(unsigned), h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     g_create_msg = std::string("init: ") + cudaGetErrorString(e);
@@ -463,12 +448,15 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
   if (tiled) {
     std::string terr;
     for (int b = 0; b < 2; ++b) {
-      const bool ok =
-          cfg->storage == LB_RT_F32
-              ? make_pop_tensor_map(&h->tmap[b], h->grid, h->Ni, h->pop[b], h->dpt, h->zc, terr)
-              : make_pop16_tensor_map(&h->tmap[b], h->grid, h->Ni, h->pop[b], cfg->storage,
-                                      h->dpt, h->zc, terr) &&
-                    make_e_tensor_map(&h->emap[b], h->grid, h->ef[b], h->zc, terr);
+      auto maps = [&](CUtensorMap* pm, CUtensorMap* em, int zc) {
+        return cfg->storage == LB_RT_F32
+                   ? make_pop_tensor_map(pm, h->grid, h->Ni, h->pop[b], h->dpt, zc, terr)
+                   : make_pop16_tensor_map(pm, h->grid, h->Ni, h->pop[b], cfg->storage, h->dpt, zc, terr) &&
+                         make_e_tensor_map(em, h->grid, h->ef[b], zc, terr);
+      };
+      const bool ok = maps(&h->tmap[b], &h->emap[b], h->zc) &&
+                      (cfg->moving || h->zc == static_flux_zc(h->dpt) ||
+                       maps(&h->tmap_flux[b], &h->emap_flux[b], static_flux_zc(h->dpt)));
       if (!ok) {
         g_create_msg = terr;
         lb_rt_destroy(h);
@@ -477,15 +465,10 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
     }
     h->tmap_ok = true;
     e = plan_static_grid(h->grid, h->Ni, h->dpt, h->zc, cfg->storage, &h->nzc, &h->ctas,
-                         cfg->moving != 0, h->pipelined);
-    if (e != cudaSuccess && h->pipelined) {
-      // the pipelined kernel cannot be resident with this plan on this
-      // device: the first-generation kernel runs the same plan
-      (void)cudaGetLastError();
-      h->pipelined = false;
-      e = plan_static_grid(h->grid, h->Ni, h->dpt, h->zc, cfg->storage, &h->nzc, &h->ctas,
-                           cfg->moving != 0, false);
-    }
+                         cfg->moving != 0);
+    if (e == cudaSuccess && !cfg->moving && h->zc != static_flux_zc(h->dpt))
+      e = plan_static_grid(h->grid, h->Ni, h->dpt, static_flux_zc(h->dpt), cfg->storage, &h->nzc_flux,
+                           &h->ctas_flux);
     if (e != cudaSuccess) {
       g_create_msg = std::string("static kernel grid: ") + cudaGetErrorString(e);
       lb_rt_destroy(h);

@@ -86,15 +86,19 @@ struct StepLaunch {
   const void* in;      // populations at t (padded layout)
   void* out;           // populations at t + dt
   const CUtensorMap* tmap_in;  // TMA descriptor of `in` (host copy)
+  // flux terms, where their boxes (static_flux_zc planes) differ, or null
+  const CUtensorMap* tmap_flux;
+  const CUtensorMap* tmap_e_flux;
+  int nzc_flux, ctas_flux;
   const CUtensorMap* tmap_e;   // 16-bit storage: TMA descriptor of the E array at t
   const float* e_in;           // 16-bit storage: E array at t (padded, float32)
   float* e_out;                // 16-bit storage: E array at t + dt (padded, float32)
   double* budget_partials;  // [nblocks][2] (sum E*, sum E_collided) or nullptr
   long long partials_cap;   // slots available; a launcher whose grid is larger refuses
   unsigned* err;            // device error word
+  unsigned* sched;          // static step: tile counter, CTAs done (2 words, zero between launches)
   float* mom_E;             // FP32 static step: E of the new state, dense [sites], or nullptr
   float* mom_F;             // FP32 static step: F of the new state, dense [3][sites], or nullptr
-  bool sc;                  // static step: the pipelined kernel (kernels_sc.cu)
 };
 
 // One problem of a static step launch.  The single-problem launch passes it
@@ -125,35 +129,23 @@ struct BatchLaunch {
   int nprob, ntiles;         // problems, total tiles
   int N, dpt, zc, storage;
   int ctas;
-  int periodic;              // some problem has a periodic axis
   int alt;                   // 1: the alternative batched kernel of this dpt (batch_alt_zc)
+  int flux;                  // some problem has lambda != 0
+  unsigned* sched;           // tile counters (4 words, zero between launches)
   unsigned* err;
 };
-cudaError_t launch_tma_static_batch(const BatchLaunch& B, const DirTable& t, cudaStream_t s);
-cudaError_t launch_tma16_static_batch(const BatchLaunch& B, const DirTable& t, cudaStream_t s);
-cudaError_t occupancy_static_batch(int storage, int dpt, int zc, int G, int* per_sm, int alt = 0);
-// Planes per batch of the alternative batched kernel compiled for this storage
-// and directions-per-warp (same memory layout, other registers / planes per
-// batch, timed by the batch autotuner against the tile plan's own kernel), or
-// 0 when there is none.
-int batch_alt_zc(int storage, int dpt);
-int batch_alt_zc16(int dpt);
+cudaError_t launch_static_batch(const BatchLaunch& B, const DirTable& t, cudaStream_t s);
+cudaError_t occupancy_static_batch(int storage, int dpt, int zc, int Ni, int* per_sm, int alt = 0);
+int batch_alt_zc(int dpt, int zc);
 // Two groups with different tile plans in ONE batched launch: group A's
 // problems run on CTAs 0 .. ctas_a - 1 of the ctas-CTA grid, group B's on the
-// rest; a block has the warps of the larger plan.  Supported for the plan
-// pairs each storage type compiles (static_batch_pair_supported); A and B in
-// that pair's order.
-bool static_batch_pair_supported(int storage, int dpt_a, int zc_a, int dpt_b, int zc_b);
+// rest; a block has the warps of the larger plan.  Supported for the 42-
+// direction plan (A) with the 162-direction one (B).
+bool static_batch_pair_supported(int dpt_a, int zc_a, int dpt_b, int zc_b);
 cudaError_t launch_static_batch_pair(const BatchLaunch& A, const DirTable& ta, const BatchLaunch& B,
                                      const DirTable& tb, int ctas_a, int ctas, cudaStream_t s);
-cudaError_t occupancy_static_batch_pair(int storage, int dpt_a, int zc_a, int ga, int dpt_b,
-                                        int zc_b, int gb, int* per_sm);
-bool tma16_pair_supported(int da, int za, int db, int zb);
-cudaError_t launch_tma16_static_batch_pair(const BatchLaunch& A, const DirTable& ta,
-                                           const BatchLaunch& B, const DirTable& tb, int ctas_a,
-                                           int ctas, cudaStream_t s);
-cudaError_t occupancy_tma16_pair(int storage, int da, int za, int ga, int db, int zb, int gb,
-                                 int* per_sm);
+cudaError_t occupancy_static_batch_pair(int storage, int dpt_a, int zc_a, int Na, int dpt_b,
+                                        int zc_b, int Nb, int* per_sm);
 
 // Kernel launchers.  Return cudaGetLastError() (or an error without
 // launching when the configuration is not supported).
@@ -186,17 +178,23 @@ cudaError_t launch_total_energy(const Grid& g, int N, const void* pop, const flo
                                 cudaStream_t s);
 
 // TMA descriptor of a padded float32 population buffer viewed as the 4D
-// tensor [PZ][PY][Ni][PX] with box (68, dpt, 2, zc) (kernels_tma.cu), and the
-// tile plans the static kernel is compiled for.
+// tensor [PZ][PY][Ni][PX] with box (68, dpt, 2, zc) (static_step.cu), and the
+// static kernel's tile plans.
 bool make_pop_tensor_map(CUtensorMap* map, const Grid& g, int Ni, void* base, int dpt, int zc,
                          std::string& err);
-extern const int kTilePlans[][3];
-extern const int kNumTilePlans;
-size_t step_tile_smem(int dpt, int zc, int warps);
-// z chunks and CTA count of the static kernel's persistent grid for this
+struct TilePlan {
+  int dpt, planes, max_warps;  // directions per warp, planes the grid must have, most warps
+};
+// lists of plans in order of preference (the next list only where none of the
+// first fits); returns the number of lists
+int static_plan_lists(int storage, const TilePlan* lists[2], int counts[2]);
+int static_zc(int dpt, const Grid& g);  // planes per batch
+int static_flux_zc(int dpt);            // the same with the flux terms
+cudaError_t occupancy_static(int storage, int dpt, int zc, int Ni, int* per_sm);
+// z chunks and CTA count of the tiled kernels' persistent grid for this
 // grid and plan on the current device (occupancy query).
 cudaError_t plan_static_grid(const Grid& g, int Ni, int dpt, int zc, int storage, int* nzc,
-                             int* ctas, bool moving = false, bool sc = false);
+                             int* ctas, bool moving = false);
 // Moving fluid, FP32 populations, TMA tiles (kernels_tma_moving.cu): one
 // plane per batch; plans (directions per warp, 1, thread cap).
 extern const int kTilePlansMoving[][3];
@@ -208,25 +206,6 @@ cudaError_t launch_tma_moving(const StepLaunch& L, const MovingCoef& c, const Di
 cudaError_t occupancy_tma16_moving(int storage, int dpt, int G, int* per_sm);
 cudaError_t launch_tma16_moving(const StepLaunch& L, const MovingCoef& c, const DirTable& t,
                                 int storage, cudaStream_t s, int* nblocks);
-// Pipelined static step (kernels_sc.cu), float32 and 16-bit storage, single
-// problem: plans (directions per warp, planes per batch, thread cap with the
-// coefficient warps); shared memory and resident CTAs per SM for
-// `stream_warps` stream warps.
-extern const int kTilePlansSC[][3];
-extern const int kNumTilePlansSC;
-size_t step_tile_smem_sc(int storage, int dpt, int zc, int stream_warps);
-cudaError_t occupancy_sc(int storage, int dpt, int zc, int stream_warps, int* per_sm);
-cudaError_t launch_sc_static(const StepLaunch& L, const StaticCoef& c, const DirTable& t, int storage,
-                             cudaStream_t s, int* nblocks);
-// 16-bit storage (kernels_tma16.cu): f_i = I_i / w_i = E (1 + q_i) with E a
-// padded float32 [PZ][PY][PX] array and q_i stored in FP16 or BF16.
-size_t step_tile_smem16(int dpt, int zc, int warps);
-extern const int kTilePlans16[][3];
-extern const int kNumTilePlans16;
-cudaError_t launch_tma16_static(const StepLaunch& L, const StaticCoef& c, const DirTable& t,
-                                int storage, cudaStream_t s, int* nblocks);
-cudaError_t occupancy_tma16(int storage, int dpt, int zc, int G, int* per_sm, bool batch = false,
-                            int alt = 0);
 bool make_pop16_tensor_map(CUtensorMap* map, const Grid& g, int Ni, void* base, int storage, int dpt,
                            int zc, std::string& err);
 bool make_e_tensor_map(CUtensorMap* map, const Grid& g, float* base, int zc, std::string& err);

@@ -1,7 +1,7 @@
 // Device helpers shared by the TMA-fed step kernels (float32 and 16-bit
 // storage): packed float32 x 2 arithmetic, mbarrier and TMA wrappers with
 // bounded waits, the static collision scalars and the persistent tile
-// schedule.  Included by kernels_tma.cu and kernels_tma16.cu only.
+// schedule.
 #pragma once
 
 #include "lb_rt_internal.h"
@@ -28,16 +28,15 @@ __device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
 }
-// One bounded try: the thread may be suspended until the phase completes or
-// about 20 microseconds pass (the hint is in nanoseconds), so a waiting warp
-// does not take issue slots from the warps that have work.
+// One bounded try.  No suspend hint: the hardware suspends the warp for a
+// while on its own; a hint is turned into a loop of sleeps.
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(20000u)
+      : "r"(bar), "r"(parity)
       : "memory");
   return ok != 0;
 }
@@ -62,7 +61,7 @@ __device__ __forceinline__ void fence_proxy_async() {
 }
 
 // CTA barrier.  A block that runs one tile plan uses __syncthreads(); a
-// block of a launch shared by two plans (kernels_tma16.cu, kernels_tma.cu)
+// block of a launch shared by two plans (k_static_pair)
 // has idle warps that leave at once, so its barriers are named barriers
 // counting the nthreads threads of the plan's warps.
 template <bool PART>
@@ -92,6 +91,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
   return true;
 }
 
+// The same with an outcome that is uniform over the (converged) warp.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, unsigned* err) {
+  if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+  const long long t0 = clock64();
+  int spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
+    if ((++spins & 63) == 0 && __any_sync(0xffffffffu, clock64() - t0 > WAIT_CYCLES)) {
+      atomicOr(err, 1u);
+      return false;
+    }
+  }
+  return true;
+}
+
 __device__ __forceinline__ float fld(const float* __restrict__ p, float s, long long i) {
   return p ? __ldg(p + i) : s;
 }
@@ -104,6 +117,13 @@ __device__ __forceinline__ void cp_async4(float* sdst, const float* gsrc) {
 }
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// wait until at most N of the thread's latest groups are outstanding
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 struct Coef {
@@ -178,12 +198,9 @@ __host__ __device__ constexpr int slot_floats() {
 struct TileGeom {
   int x0, y, zbeg, zlen;
 };
-// rot: the x-blocks of the tile's row are permuted cyclically by rot (the
-// same rot for every tile of a row keeps the map a bijection).
-__device__ __forceinline__ TileGeom tile_geom(int ti, int nxb, int ny, int nz, int nzc,
-                                              int rot = 0) {
+__device__ __forceinline__ TileGeom tile_geom(int ti, int nxb, int ny, int nz, int nzc) {
   TileGeom tg;
-  tg.x0 = ((ti % nxb + rot) % nxb) * 64;
+  tg.x0 = ti % nxb * 64;
   const int r = ti / nxb;
   tg.y = r % ny;
   const int c = r / ny;
@@ -198,18 +215,6 @@ __device__ __forceinline__ TileGeom tile_geom(int ti, int nxb, int ny, int nz, i
 // the output plane z = zbeg - 1 + m ZC + j (for both signs of n^z, with the
 // box shifted by one plane for sgn n^z = -1), which is stored when it lies in
 // the tile; the first plane of a tile only seeds the carried value.
-// Rotation of the x-blocks for tile ti (problem-relative) of a persistent
-// grid of ncta CTAs.  When ncta is a multiple of the x-blocks per row, CTA b
-// would keep one x-block for the whole step; with a periodic x axis the CTAs
-// of the first and last x-block also write the ghost columns and fall
-// behind.  Rotating the x-blocks of every row by the round ti / ncta makes
-// every CTA walk all x-blocks, while the tiles of one round (and so the
-// neighbouring rows in flight together) stay the same.  A row never spans
-// two rounds because ncta is a multiple of nxb.
-__device__ __forceinline__ int tile_rot(int ti, int nxb, int ncta, bool periodic_x) {
-  return (periodic_x && nxb > 1 && ncta % nxb == 0) ? ti / ncta : 0;
-}
-
 template <int ZC>
 __device__ __forceinline__ int tile_items(int zlen) {
   return (zlen + 1 + ZC - 1) / ZC;
