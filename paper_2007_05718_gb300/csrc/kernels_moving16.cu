@@ -63,7 +63,6 @@ __device__ __forceinline__ void store_e(float* e, const Grid& g, int z, int y, i
 // q = (A f* + g' src) / E^' - 1.  One plane per batch.
 struct DirConstM16 {
   float4 s0, s1, s2, s3;  // (a_x, a_y), (a_z', n_x), (n_y, n_z), (w, dt) pairs
-  int sh, inert, pad0, pad1;
 };
 
 template <class ST, bool PER, int DPT, int R, int MAXT, int REGS>
@@ -116,9 +115,6 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
     d.s1 = make_float4(azw, azw, nw.x, nw.x);
     d.s2 = make_float4(nw.y, nw.y, nw.z, nw.z);
     d.s3 = make_float4(nw.w, nw.w, dt, dt);
-    d.sh = (oct & 1) ? 1 : -1;
-    d.inert = oct & 8;
-    d.pad0 = d.pad1 = 0;
     dirs[i] = d;
   }
   if (lane == 0) {
@@ -156,9 +152,11 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
-  unsigned inert_mask = 0;
-#pragma unroll
-  for (int k = 0; k < DPT; ++k) inert_mask |= dirs[i0 + k].inert ? 1u << k : 0u;
+  // padding and x-negative directions of the warp (from votes, so that branches
+  // on them are known to be uniform)
+  const int oct_l = lane < DPT ? __float_as_int(t.au[i0 + lane].w) : 8;
+  const unsigned inert_mask = __ballot_sync(0xffffffffu, lane < DPT && (oct_l & 8));
+  const unsigned xneg_mask = __ballot_sync(0xffffffffu, oct_l & 1);
 
   unsigned char* my_ring = ring + (size_t)g * R * SLOTB;
   bool alive = true;
@@ -275,9 +273,9 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
                                 f2fma(vy, make_float2(s2.x, s2.y), f2mul(vx, make_float2(s1.z, s1.w))));
         beta = f2sub(one2, vn);
         const float2 den = f2fma(cA, beta, one2);
-        A = make_float2(__fdividef(1.f, den.x), __fdividef(1.f, den.y));
+        A = f2rcp(den);
         const float2 wb = f2mul(W, beta);
-        const float2 iw = make_float2(__fdividef(1.f, wb.x), __fdividef(1.f, wb.y));
+        const float2 iw = f2rcp(wb);
         gp = f2mul(f2mul(A, make_float2(s3.z, s3.w)), f2mul(iw, f2mul(iw, iw)));
       };
       while (issued < q + R && issue()) {
@@ -291,7 +289,10 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
       const float2 EPo = *reinterpret_cast<const float2*>(eo);
       const float2 EPu = *reinterpret_cast<const float2*>(eu);
       const float Emo = eo[-1], Epo = eo[2], Emu = eu[-1], Epu = eu[2];
-      float2 Is[DPT];  // f*_i
+      // A_i f*_i and g'_i of the item, where the registers hold both; otherwise
+      // f*_i, and the store forms A_i and g'_i again
+      constexpr bool KEEP = DPT <= 5 || REGS >= 128;
+      float2 Is[DPT], Gk[KEEP ? DPT : 1];
       float2 aS = make_float2(0.f, 0.f), aX = aS, aY = aS, aA = aS, aG = aS;
 #pragma unroll
       for (int k = 0; k < DPT; ++k) {
@@ -306,22 +307,27 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
         const float2 fo = f2fma(EPo, qo, EPo);
         const float2 fu = f2fma(EPu, qu, EPu);
         float2 So, Su;
-        if (d.sh > 0) {
-          So = make_float2(fo.y, fmaf(Epo, C2::to1(po[2]), Epo));
-          Su = make_float2(fu.y, fmaf(Epu, C2::to1(pu[2]), Epu));
+        if (xneg_mask >> k & 1u) {
+          So = make_float2(fo.y - fo.x, fmaf(Epo, C2::to1(po[2]), Epo) - fo.y);
+          Su = make_float2(fu.y - fu.x, fmaf(Epu, C2::to1(pu[2]), Epu) - fu.y);
         } else {
-          So = make_float2(fmaf(Emo, C2::to1(po[-1]), Emo), fo.x);
-          Su = make_float2(fmaf(Emu, C2::to1(pu[-1]), Emu), fu.x);
+          So = make_float2(fmaf(Emo, C2::to1(po[-1]), Emo) - fo.x, fo.x - fo.y);
+          Su = make_float2(fmaf(Emu, C2::to1(pu[-1]), Emu) - fu.x, fu.x - fu.y);
         }
-        const float2 X0 = f2fma(ax, f2sub(So, fo), fo);
-        const float2 X1 = f2fma(ax, f2sub(Su, fu), fu);
+        const float2 X0 = f2fma(ax, So, fo);
+        const float2 X1 = f2fma(ax, Su, fu);
         const float2 Bn = f2fma(ay, f2sub(X1, X0), X0);
         const float2 r = f2fma(az, f2sub(carry[k], Bn), Bn);
         carry[k] = Bn;
-        Is[k] = r;
         float2 beta, A, gp;
         coll(d, beta, A, gp);
         const float2 af = f2mul(A, r);
+        if constexpr (KEEP) {
+          Is[k] = af;
+          Gk[k] = gp;
+        } else {
+          Is[k] = r;
+        }
         const float2 wb2 = f2mul(w2, f2mul(beta, beta));
         aS = f2fma(w2, r, aS);
         aX = f2fma(wb2, f2fma(gp, et, af), aX);
@@ -385,15 +391,23 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
                         !(y_face && ny == 1) && !(zface && nz == 1);
       const bool xghost = __any_sync(0xffffffffu, gx_lo || gx_hi);
       const int yface_rows = (y == ny - 1 ? 0 : ny + 1) - (y + 1);
+      auto value = [&](int k) -> T2 {
+        float2 o;
+        if constexpr (KEEP) {
+          o = f2fma(Gk[k], src, Is[k]);
+        } else {
+          float2 beta, A, gp;
+          coll(dirs[i0 + k], beta, A, gp);
+          o = f2fma(gp, src, f2mul(A, Is[k]));
+        }
+        return C2::from2(f2fma(o, rinv, make_float2(-1.f, -1.f)));
+      };
       if (alive && fast) {
         ST* base = orow + (long long)(z + 1) * gr.sz;
 #pragma unroll
         for (int k = 0; k < DPT; ++k) {
           if (inert_mask >> k & 1u) continue;
-          float2 beta, A, gp;
-          coll(dirs[i0 + k], beta, A, gp);
-          const float2 qn = f2fma(f2fma(gp, src, f2mul(A, Is[k])), rinv, make_float2(-1.f, -1.f));
-          const T2 hq = C2::from2(qn);
+          const T2 hq = value(k);
           ST* dst = base + (long long)k * gr.si;
           if constexpr (!PER) {
             *reinterpret_cast<T2*>(dst) = hq;
@@ -412,15 +426,24 @@ k_step_moving16(const __grid_constant__ CUtensorMap tmap, const __grid_constant_
           }
         }
       } else if (alive && in0 && zok) {
+        // partial tile or an extent of 1 on a periodic axis: the site and every
+        // mirror row / plane, and the ghost columns
+#pragma unroll 1
+        for (int im = 0; im < 9; ++im) {
+          const int iy = im % 3, iz = im / 3;
+          const int row = iy == 0 ? y + 1 : !gr.periodic[1] ? -1 : iy == 1 ? (y == ny - 1 ? 0 : -1) : (y == 0 ? ny + 1 : -1);
+          const int pl = iz == 0 ? z + 1 : !gr.periodic[2] ? -1 : iz == 1 ? (z == nz - 1 ? 0 : -1) : (z == 0 ? nz + 1 : -1);
+          if (row < 0 || pl < 0) continue;
+          ST* dst = out + (long long)i0 * gr.si + (long long)pl * gr.sz + (long long)row * gr.sy + xa + GL;
 #pragma unroll
-        for (int k = 0; k < DPT; ++k) {
-          if (inert_mask >> k & 1u) continue;
-          float2 beta, A, gp;
-          coll(dirs[i0 + k], beta, A, gp);
-          const float2 qn = f2fma(f2fma(gp, src, f2mul(A, Is[k])), rinv, make_float2(-1.f, -1.f));
-          const T2 hq = C2::from2(qn);
-          store_pop(out, gr, i0 + k, z, y, xa, hq.x);
-          if (in1) store_pop(out, gr, i0 + k, z, y, xa + 1, hq.y);
+          for (int k = 0; k < DPT; ++k, dst += gr.si) {
+            if (inert_mask >> k & 1u) continue;
+            const T2 h = value(k);
+            if (in1) *reinterpret_cast<T2*>(dst) = h;
+            else dst[0] = h.x;
+            if (gx_lo) dst[GL - 1 - (xa + GL)] = lo_from_y ? h.y : h.x;
+            if (gx_hi) dst[nx - xa] = h.x;
+          }
         }
       }
     }

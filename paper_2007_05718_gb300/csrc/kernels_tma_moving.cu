@@ -27,17 +27,12 @@ using namespace tma;
 
 // Per-direction constants as pre-broadcast pairs: s0 = (a_x, a_x, a_y, a_y),
 // s1 = (a_z', a_z', n_x, n_x), s2 = (n_y, n_y, n_z, n_z), s3 = (dt w, dt w,
-// -, -); sh = offset of the x-upwind pair; inert = padding entry.
+// -, -).
 struct DirConstM {
   float4 s0, s1, s2, s3;
-  int sh, inert, pad0, pad1;
 };
 
 constexpr int kQ = 5;  // partial quantities: sum I*, X, Y, sum A I*, sum g
-
-__device__ __forceinline__ float2 f2rcp(float2 a) {
-  return make_float2(__fdividef(1.f, a.x), __fdividef(1.f, a.y));
-}
 
 template <bool PER, int DPT, int R, int MAXT, int REGS>
 __global__ void __launch_bounds__(MAXT) __maxnreg__(REGS)
@@ -85,9 +80,6 @@ k_step_moving_tma(const __grid_constant__ CUtensorMap tmap, const StepLaunch L,
     d.s1 = make_float4(azw, azw, nw.x, nw.x);
     d.s2 = make_float4(nw.y, nw.y, nw.z, nw.z);
     d.s3 = make_float4(dt * nw.w, dt * nw.w, 0.f, 0.f);
-    d.sh = (oct & 1) ? 1 : -1;
-    d.inert = oct & 8;
-    d.pad0 = d.pad1 = 0;
     dirs[i] = d;
   }
   if (lane == 0)
@@ -122,9 +114,11 @@ k_step_moving_tma(const __grid_constant__ CUtensorMap tmap, const StepLaunch L,
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
-  unsigned inert_mask = 0;
-#pragma unroll
-  for (int k = 0; k < DPT; ++k) inert_mask |= dirs[i0 + k].inert ? 1u << k : 0u;
+  // padding and x-negative directions of the warp (from votes, so that branches
+  // on them are known to be uniform)
+  const int oct_l = lane < DPT ? __float_as_int(t.au[i0 + lane].w) : 8;
+  const unsigned inert_mask = __ballot_sync(0xffffffffu, lane < DPT && (oct_l & 8));
+  const unsigned xneg_mask = __ballot_sync(0xffffffffu, oct_l & 1);
 
   float* my_ring = ring + (size_t)g * R * SLOT;
   bool alive = true;
@@ -242,7 +236,11 @@ k_step_moving_tma(const __grid_constant__ CUtensorMap tmap, const StepLaunch L,
       float* slot = my_ring + (size_t)(q % R) * SLOT;
       const float* own = slot + row_own * DPT * BOXX + wc;
       const float* up = slot + row_up * DPT * BOXX + wc;
-      float2 Is[DPT];
+      // A_i I*_i and g_i of the item, where the registers hold both; otherwise
+      // I*_i, and the store forms A_i and g_i again (8 instead of 4 reciprocals
+      // a pair, whose unit is then the busiest)
+      constexpr bool KEEP = DPT <= 5 || REGS >= 128;
+      float2 Is[DPT], Gk[KEEP ? DPT : 1];
       float2 aS = make_float2(0.f, 0.f), aX = aS, aY = aS, aA = aS, aG = aS;
 #pragma unroll
       for (int k = 0; k < DPT; ++k) {
@@ -256,22 +254,27 @@ k_step_moving_tma(const __grid_constant__ CUtensorMap tmap, const StepLaunch L,
         // the x-upwind pair shares one value with the lane's own pair; one
         // 4-byte load completes it (the x sign is uniform over the warp)
         float2 S0, S1;
-        if (d.sh > 0) {
-          S0 = make_float2(P0.y, own[off + 2]);
-          S1 = make_float2(P1.y, up[off + 2]);
+        if (xneg_mask >> k & 1u) {
+          S0 = make_float2(P0.y - P0.x, own[off + 2] - P0.y);
+          S1 = make_float2(P1.y - P1.x, up[off + 2] - P1.y);
         } else {
-          S0 = make_float2(own[off - 1], P0.x);
-          S1 = make_float2(up[off - 1], P1.x);
+          S0 = make_float2(own[off - 1] - P0.x, P0.x - P0.y);
+          S1 = make_float2(up[off - 1] - P1.x, P1.x - P1.y);
         }
-        const float2 X0 = f2fma(ax, f2sub(S0, P0), P0);
-        const float2 X1 = f2fma(ax, f2sub(S1, P1), P1);
+        const float2 X0 = f2fma(ax, S0, P0);
+        const float2 X1 = f2fma(ax, S1, P1);
         const float2 Bn = f2fma(ay, f2sub(X1, X0), X0);
         const float2 r = f2fma(az, f2sub(carry[k], Bn), Bn);
         carry[k] = Bn;
-        Is[k] = r;
         float2 beta, A, gg;
         coll(d, beta, A, gg);
         const float2 ai = f2mul(A, r);
+        if constexpr (KEEP) {
+          Is[k] = ai;
+          Gk[k] = gg;
+        } else {
+          Is[k] = r;
+        }
         const float2 b2 = f2mul(beta, beta);
         aS = f2add(aS, r);
         aX = f2fma(b2, f2fma(gg, et, ai), aX);
@@ -331,14 +334,18 @@ k_step_moving_tma(const __grid_constant__ CUtensorMap tmap, const StepLaunch L,
                         !(y_face && ny == 1) && !(zface && nz == 1);
       const bool xghost = __any_sync(0xffffffffu, gx_lo || gx_hi);
       const int yface_rows = (y == ny - 1 ? 0 : ny + 1) - (y + 1);
+      auto value = [&](int k) -> float2 {
+        if constexpr (KEEP) return f2fma(Gk[k], src, Is[k]);
+        float2 beta, A, gg;
+        coll(dirs[i0 + k], beta, A, gg);
+        return f2fma(gg, src, f2mul(A, Is[k]));
+      };
       if (alive && fast) {
         float* base = orow + (long long)(z + 1) * gr.sz;
 #pragma unroll
         for (int k = 0; k < DPT; ++k) {
           if (inert_mask >> k & 1u) continue;
-          float2 beta, A, gg;
-          coll(dirs[i0 + k], beta, A, gg);
-          const float2 o = f2fma(gg, src, f2mul(A, Is[k]));
+          const float2 o = value(k);
           float* dst = base + (long long)k * gr.si;
           if constexpr (!PER) {
             *reinterpret_cast<float2*>(dst) = o;
@@ -357,15 +364,24 @@ k_step_moving_tma(const __grid_constant__ CUtensorMap tmap, const StepLaunch L,
           }
         }
       } else if (alive && in0 && zok) {
-        // partial tile or an extent of 1 on a periodic axis: every image
+        // partial tile or an extent of 1 on a periodic axis: the site and every
+        // mirror row / plane, and the ghost columns
+#pragma unroll 1
+        for (int im = 0; im < 9; ++im) {
+          const int iy = im % 3, iz = im / 3;
+          const int row = iy == 0 ? y + 1 : !gr.periodic[1] ? -1 : iy == 1 ? (y == ny - 1 ? 0 : -1) : (y == 0 ? ny + 1 : -1);
+          const int pl = iz == 0 ? z + 1 : !gr.periodic[2] ? -1 : iz == 1 ? (z == nz - 1 ? 0 : -1) : (z == 0 ? nz + 1 : -1);
+          if (row < 0 || pl < 0) continue;
+          float* dst = out + (long long)i0 * gr.si + (long long)pl * gr.sz + (long long)row * gr.sy + xa + GL;
 #pragma unroll
-        for (int k = 0; k < DPT; ++k) {
-          if (inert_mask >> k & 1u) continue;
-          float2 beta, A, gg;
-          coll(dirs[i0 + k], beta, A, gg);
-          const float2 o = f2fma(gg, src, f2mul(A, Is[k]));
-          store_pop(out, gr, i0 + k, z, y, xa, o.x);
-          if (in1) store_pop(out, gr, i0 + k, z, y, xa + 1, o.y);
+          for (int k = 0; k < DPT; ++k, dst += gr.si) {
+            if (inert_mask >> k & 1u) continue;
+            const float2 o = value(k);
+            if (in1) *reinterpret_cast<float2*>(dst) = o;
+            else dst[0] = o.x;
+            if (gx_lo) dst[GL - 1 - (xa + GL)] = lo_from_y ? o.y : o.x;
+            if (gx_hi) dst[nx - xa] = o.x;
+          }
         }
       }
     }
