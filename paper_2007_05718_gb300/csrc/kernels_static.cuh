@@ -230,6 +230,16 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
 
   auto flat_of = [&](const ProblemDesc& D) { return ZC == 1 && D.g.dims == 2; };
 
+  // byte offsets of the lane's data in shared memory, kept in registers (left
+  // to itself the compiler forms them again for every batch)
+  int off_own = L::RING + g * kRing * SLOT + (row_own * DPT * BOX + 2 + 2 * lane) * (int)sizeof(ST);
+  int off_up = L::RING + g * kRing * SLOT + (row_up * DPT * BOX + 2 + 2 * lane) * (int)sizeof(ST);
+  int off_dirs = L::DIRS + i0 * (int)sizeof(DirC<FLUX>);
+  int off_eo = L::ERING + ((zs * 3 + 1) * kBoxE + 2 + 2 * lane) * 4;
+  int off_eu = L::ERING + ((zs * 3 + erow_up) * kBoxE + 2 + 2 * lane) * 4;
+  asm volatile("" : "+r"(off_own), "+r"(off_up), "+r"(off_dirs), "+r"(off_eo), "+r"(off_eu));
+  const DirC<FLUX>* const my_dirs = reinterpret_cast<const DirC<FLUX>*>(smem_raw + off_dirs);
+
   // ---- tiles of this CTA ------------------------------------------------------
   // Tile number 0 is tile `cta` of the list; the next ones are taken from a
   // counter (sched[0]) as the CTA comes to them, so that at any time the tiles
@@ -544,7 +554,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     }
     // float32: I' = alpha I* + w c0 + (w n) . c1; 16 bits: q' = A' f* + c0' + n . c1'
     auto value = [&](int k, int j) -> float2 {
-      const DirC<FLUX>& d = dirs[i0 + k];
+      const DirC<FLUX>& d = my_dirs[k];
       float2 eq;
       if constexpr (F32) {
         const float4 b = d.b;
@@ -656,25 +666,22 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
 #pragma unroll
   for (int k = 0; k < DPT; ++k) carry[k] = make_float2(0.f, 0.f);
   BatchCtx<ST> ctx{};  // batch whose store is pending
-  const int wc = 2 + 2 * lane;  // box column of the lane's pair
 
   // stream directions K0 .. K1 - 1 of batch q into dst[0 ..], adding to the
   // partial moments
   auto stream = [&](auto K0_, auto K1_, int q, float2 (*dst)[ZC], float2 (&aE)[ZC], float2 (&aX)[ZC],
                     float2 (&aY)[ZC], float2 (&aZ)[ZC]) {
     constexpr int K0 = decltype(K0_)::value, K1 = decltype(K1_)::value;
-    const unsigned char* slot = my_ring + (size_t)(q % kRing) * SLOT;
-    const ST* own = reinterpret_cast<const ST*>(slot) + row_own * DPT * BOX + wc;
-    const ST* up = reinterpret_cast<const ST*>(slot) + row_up * DPT * BOX + wc;
+    const ST* own = reinterpret_cast<const ST*>(smem_raw + off_own + q % kRing * SLOT);
+    const ST* up = reinterpret_cast<const ST*>(smem_raw + off_up + q % kRing * SLOT);
     // 16-bit storage: E^ of the lane's pair and its x-neighbours, both rows
     float2 EPo[ZC], EPu[ZC];
     float Emo[ZC], Epo[ZC], Emu[ZC], Epu[ZC];
     if constexpr (!F32) {
-      const float* es = ering + (size_t)(q % kEring) * ESLOT;
 #pragma unroll
       for (int j = 0; j < ZC; ++j) {
-        const float* eo = es + ((j + zs) * 3 + 1) * kBoxE + wc;
-        const float* eu = es + ((j + zs) * 3 + erow_up) * kBoxE + wc;
+        const float* eo = reinterpret_cast<const float*>(smem_raw + off_eo + q % kEring * (ESLOT * 4)) + j * 3 * kBoxE;
+        const float* eu = reinterpret_cast<const float*>(smem_raw + off_eu + q % kEring * (ESLOT * 4)) + j * 3 * kBoxE;
         EPo[j] = *reinterpret_cast<const float2*>(eo);
         EPu[j] = *reinterpret_cast<const float2*>(eu);
         Emo[j] = eo[-1];
@@ -685,7 +692,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     }
 #pragma unroll
     for (int k = K0; k < K1; ++k) {
-      const DirC<FLUX>& d = dirs[i0 + k];
+      const DirC<FLUX>& d = my_dirs[k];
       const float4 ca = d.a, cb = d.b;
       const float2 ax = make_float2(ca.x, ca.y), ay = make_float2(ca.z, ca.w);
       const float2 az = make_float2(cb.x, cb.y), w2 = make_float2(cb.z, cb.w);
