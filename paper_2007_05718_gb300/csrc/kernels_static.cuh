@@ -10,12 +10,14 @@
 //
 // Tiles.  A CTA owns 64 consecutive x sites of one row over a chunk of planes
 // (3D), or of a chunk of rows (2D: no direction leaves the plane, so the march
-// is along y and no seed plane is loaded); each lane owns an x-pair (packed
-// float32 x 2 arithmetic).  Warp g owns the DPT directions g DPT .. of the
-// internal order, all of one upwind (row, plane) class; per batch of ZC planes
-// one TMA box brings its directions x own and upwind row x ZC planes.  The
-// bilinear value of a plane is lerped in z against the one carried in
-// registers from the plane before, so every plane is loaded once per tile.
+// is along y, no seed plane is loaded and the mirror planes of a periodic z
+// axis, which no pull reads, are not written: two thirds of the stores); each
+// lane owns an x-pair (packed float32 x 2 arithmetic).  Warp g owns the DPT
+// directions g DPT .. of the internal order, all of one upwind (row, plane)
+// class; per batch of ZC planes one TMA box brings its directions x own and
+// upwind row x ZC planes.  The bilinear value of a plane is lerped in z against
+// the one carried in registers from the plane before, so every plane is loaded
+// once per tile.
 //
 // Who waits for whom.  The collision of a site needs the sum over all
 // directions, that is over all warps.  A warp does not wait for the sum of the
@@ -40,6 +42,18 @@
 // depend on the flux: c1 = dt kappa_0 lambda F = 0.  FLUX == false leaves out
 // the flux partials and the n . c1 terms (they are exact zeros), about a third
 // of the packed arithmetic and most of the direction constants.
+//
+// What bounds it.  float32, 256 x 256 x 64 periodic, 162 directions: 1.24 ms,
+// 3.6 GB read and 2.9 GB written in DRAM, 5.2 TB/s; 64 instructions per
+// direction and 64-site plane, issue slots 49 % busy.  Behind DRAM the
+// shared-memory wavefronts of the stream (48 of 59 cycles per direction-plane
+// with resident boxes) are the next limit.  16 bits: the decode and the lerps,
+// 84 instructions, issue slots 70 % busy, 1.16 ms.  Before (partials and
+// scalars between two CTA barriers per plane, tiles dealt out in advance) the
+// same grid took 2.0 and 2.2 ms; step times in ms:
+//   256^3 x 162 float32 7.8 -> 5.0, 16 bits 9.0 -> 4.3
+//   128^3 x 42 float32 0.21 -> 0.16, float16 0.26 -> 0.18
+//   512^2 x 162 float32 sweep 73 -> 12.6 (27 before the mirror planes went)
 //
 // Every wait is bounded (about 2 s): one that gives up sets the error word,
 // and the warp goes on with stale (in-bounds) data, still arriving at every
@@ -277,7 +291,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
         y = flat ? tg.zbeg : tg.y;
         z = flat ? 1 : tg.zbeg;
         len = flat ? -tg.zlen : tg.zlen;
-        fl = (x0 + 64 <= gr.nx ? 0 : 2) | (gr.periodic[1] || gr.periodic[2] ? 8 : 0) |
+        fl = (x0 + 64 <= gr.nx ? 0 : 2) | (gr.periodic[1] || (gr.periodic[2] && !flat) ? 8 : 0) |
              (gr.periodic[0] && (x0 == 0 || x0 + 64 >= gr.nx) ? 16 : 0);
         if constexpr (BATCH) {
           const int* src = reinterpret_cast<const int*>(&D);
@@ -346,7 +360,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     const ProblemDesc& D = desc(tn & 3);
     t_zf0 = t_zf1 = -9;
     if (t_fl & 8) {  // some axis of y, z is periodic: faces have mirrors
-      if (D.g.periodic[2]) t_zf0 = 1 - t_z, t_zf1 = D.g.nz - t_z;
+      if (t_len > 0 && D.g.periodic[2]) t_zf0 = 1 - t_z, t_zf1 = D.g.nz - t_z;
       if (t_len > 0 && D.g.periodic[1] && (t_y == 0 || t_y == D.g.ny - 1)) t_fl |= 4;
     }
     t_base = static_cast<ST*>(D.out) + (long long)i0 * D.g.si + (long long)t_z * D.g.sz +
@@ -521,11 +535,13 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
       if constexpr (!F32) {
         {
           float* e = D.e_out;
-          if (has_mirror(gr, z, y, x)) {
+          const int pz = gr.periodic[2] && !flat_of(D);
+          if ((gr.periodic[0] && (x == 0 || x == gr.nx - 1)) || (gr.periodic[1] && (y == 0 || y == gr.ny - 1)) ||
+              (pz && (z == 0 || z == gr.nz - 1))) {
             int xs[3], ys[3], zs_[3];
             const int nxs = mirrors(x, gr.nx, gr.periodic[0], GL, xs);
             const int nys = mirrors(y, gr.ny, gr.periodic[1], 1, ys);
-            const int nzs = mirrors(z, gr.nz, gr.periodic[2], 1, zs_);
+            const int nzs = mirrors(z, gr.nz, pz, 1, zs_);
             for (int a = 0; a < nzs; ++a)
               for (int b = 0; b < nys; ++b)
                 for (int cx = 0; cx < nxs; ++cx)

@@ -765,6 +765,14 @@ size_t lb_rt_state_bytes(const lb_rt* h) {
   return b;
 }
 
+// The static step does not write the mirror planes of a 2D grid's periodic z
+// axis; a saved state holds them, as copies of the one plane between them.
+static void fill_mirror_planes(const lb_rt* h, char* arr, size_t plane) {
+  if (h->cfg.dims != 2 || !h->grid.periodic[2]) return;
+  std::memcpy(arr, arr + plane, plane);
+  std::memcpy(arr + 2 * plane, arr + plane, plane);
+}
+
 lb_rt_status lb_rt_save_state(lb_rt* h, void* buf, size_t bytes) {
   if (!h || !buf) return fail(h, LB_RT_EINVAL, "null argument");
   if (bytes < lb_rt_state_bytes(h)) return fail(h, LB_RT_EINVAL, "buffer too small");
@@ -779,7 +787,12 @@ lb_rt_status lb_rt_save_state(lb_rt* h, void* buf, size_t bytes) {
     p += h->ef_bytes;
   }
   CK(h, cudaMemcpyAsync(p, h->acc, 8 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  return lb_rt_sync(h);
+  const lb_rt_status st = lb_rt_sync(h);
+  if (st != LB_RT_OK) return st;
+  p = static_cast<char*>(buf) + 64;
+  fill_mirror_planes(h, p, (size_t)h->grid.sz * elem_bytes(h->cfg.storage));
+  if (h->ef[0]) fill_mirror_planes(h, p + h->pop_bytes, h->ef_bytes / 3);
+  return LB_RT_OK;
 }
 
 lb_rt_status lb_rt_restore_state(lb_rt* h, const void* buf, size_t bytes) {

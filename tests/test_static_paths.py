@@ -91,3 +91,25 @@ def test_batch_of_uneven_grids_agrees_with_single_problems(cuda, storage, lam):
         finally:
             lbrt.lb_rt_destroy(h)
         assert np.array_equal(E, E1) and np.array_equal(F, F1)
+
+
+@pytest.mark.parametrize("storage", [F32, F16])
+@pytest.mark.parametrize("shape", [(1, 5, 63), (1, 17, 130)])
+def test_saved_state_of_a_2d_grid_holds_the_z_mirrors(shape, storage):
+    """The step leaves out the mirror planes of a 2D grid's periodic z axis; a
+    saved state has them all the same: three equal planes per array."""
+    nz, ny, nx = shape
+    h = lbrt.lb_rt_create(2, nx, ny, nz, storage=storage, bc=(P, V, P), **RING(12))
+    try:
+        lbrt.lb_rt_set_fluid(h, kappa_a=2.0, eta=1.0)
+        lbrt.lb_rt_set_state(h, W.random_populations(12, shape, 3))
+        lbrt.lb_rt_step(h, 3)
+        raw = np.frombuffer(lbrt.lb_rt_save_state(h), np.uint8)
+    finally:
+        lbrt.lb_rt_destroy(h)
+    body = raw[64:-64]
+    row = (nx + 3 + 7) // 8 * 8  # sites of a padded row
+    e_bytes = 0 if storage == F32 else 3 * 4 * row * (ny + 2)
+    for a in (body[:body.size - e_bytes], body[body.size - e_bytes:]):
+        planes = a.reshape(3, -1)
+        assert np.array_equal(planes[0], planes[1]) and np.array_equal(planes[2], planes[1])
