@@ -424,7 +424,8 @@ __global__ void k_total_partials16(Grid g, int N, const ST* __restrict__ pop,
 // the lab components of the four-vector (kt_a J - eta_t) u^mu + kt H^mu, with
 // H^0 = v.H the time component of the comoving flux (H^mu u_mu = 0,
 // signature -+++).  ST = float: populations; 16-bit types: the deviation
-// form against the E array `e`.
+// form against the E array `e`.  Two sites a thread, bound by the latency of
+// the loads at small grids: 64^3 x 42 float32, 20.7 -> 15.0 us.
 template <class ST>
 __global__ void k_coupling(Grid g, int N, const ST* __restrict__ pop, const float* __restrict__ e,
                            const __grid_constant__ DirTable t, MovingCoef c, float* __restrict__ Jo,

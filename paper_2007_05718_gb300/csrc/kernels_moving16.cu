@@ -3,6 +3,10 @@
 // and the mixed-frame equation of App. B; the storage format (E in float32 and
 // the relative deviation q_i = I_i / (w_i E) - 1 in 16 bits) is that of
 // kernels_static.cuh, the tile pipeline that of kernels_tma_moving.cu.
+//
+// What bounds it: instruction issue (16-bit decode and encode on top of the
+// float32 kernel's arithmetic), not memory.  Hardware reciprocals and products
+// kept for the store: 128^3 x 162 float16, 1.72 -> 1.37 ms.
 #include <algorithm>
 
 #include "lb_rt_internal.h"

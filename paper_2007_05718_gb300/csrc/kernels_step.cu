@@ -16,9 +16,6 @@
 
 namespace lbrt {
 
-cudaError_t launch_tma_static(const StepLaunch& L, const StaticCoef& c, const DirTable& t,
-                              int dpt, int zc, cudaStream_t s, int* nblocks);
-
 namespace {
 
 constexpr int TY = 4;  // sites per CTA along y (32 along x)

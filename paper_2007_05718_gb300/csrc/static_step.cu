@@ -37,8 +37,9 @@ int static_plan_lists(int storage, const TilePlan* lists[2], int counts[2]) {
 
 // Planes per batch of the plan's kernel.  5 directions per warp work two
 // planes a batch, which halves the per-batch work of a warp (128^3 x 42
-// sphere, float16: 0.228 -> 0.175 ms a step); the flux terms leave no registers for that, and a 2D grid has
-// one plane.
+// sphere, float16: 0.228 -> 0.175 ms a step).  The flux terms leave no
+// registers for that (64^3 x 42 with kappa_1: two planes took 1.4 times the
+// time of the kernel before, one plane 0.95), and a 2D grid has one plane.
 int static_zc(int dpt, const Grid& g) { return dpt == 5 && g.dims == 3 && g.nz >= 2 ? 2 : 1; }
 int static_flux_zc(int) { return 1; }
 
@@ -109,6 +110,8 @@ cudaError_t launch_step_static(const StepLaunch& L, const StaticCoef& c, const D
   if (L.budget_partials && k.ctas > L.partials_cap) return cudaErrorInvalidValue;
   if (nblocks) *nblocks = k.ctas;
   k.err = L.err;
+  // the budget's per-CTA partial sums want a fixed assignment of tiles to CTAs;
+  // otherwise the counter (256^3 x 162 float32: 9.2 ms dealt out, 5.7 counted)
   k.sched = L.budget_partials ? nullptr : L.sched;
   k.dirs = &t;
   k.stream = s;

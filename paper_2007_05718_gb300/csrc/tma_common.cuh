@@ -200,12 +200,13 @@ __host__ __device__ constexpr int slot_floats() {
   return ((BOXX * DPT * 2 * ZC * 4 + 127) / 128) * 32;  // 128-byte aligned slots
 }
 
-// Tile schedule of the persistent grid: tile ti covers the 64 columns
+// Tile schedule of the persistent grids: tile ti covers the 64 columns
 // x0 .. x0 + 63 of row y over the planes zbeg .. zbeg + zlen - 1; tiles are
-// numbered x-block fastest, then y, then z chunk, and CTA b takes tiles b,
-// b + gridDim.x, ...  so that the tiles in flight at one time are
-// neighbouring rows whose shared upwind rows meet in L2.  The nz planes are
-// split into nzc chunks of near-equal length.
+// numbered x-block fastest, then y, then z chunk, and taken in that order (the
+// moving step: CTA b takes b, b + gridDim.x, ...; the static step: from a
+// counter), so that the tiles in flight at one time are neighbouring rows whose
+// shared upwind rows meet in L2.  The nz planes are split into nzc chunks of
+// near-equal length.
 struct TileGeom {
   int x0, y, zbeg, zlen;
 };
