@@ -267,7 +267,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
   // Warp 0 takes tile n + 1 when it opens tile n and publishes its geometry in
   // the queue (slot n + 1 mod 4) while it works on the tile's first item.
   volatile TileInfo* const tq = reinterpret_cast<volatile TileInfo*>(smem_raw + L::TILEQ);
-  volatile int* const tq_count = reinterpret_cast<volatile int*>(tq + 4);
+  const uint32_t tq_count = smem0 + L::TILEQ + 4 * (int)sizeof(TileInfo);
   ProblemDesc* const pd = reinterpret_cast<ProblemDesc*>(smem_raw + L::DESC);
   auto desc = [&](int slot) -> const ProblemDesc& { return BATCH ? pd[slot] : one; };
   int w_prob = 0;  // warp 0: problem of the tile published last
@@ -297,8 +297,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
           const int* src = reinterpret_cast<const int*>(&D);
           int* dst = reinterpret_cast<int*>(&pd[n & 3]);
           for (int w = lane; w < (int)(sizeof(ProblemDesc) / 4); w += 32) dst[w] = src[w];
-          __threadfence_block();
-          __syncwarp();
+          __syncwarp();  // orders the lanes' copies before lane 0's release
         }
       }
     }
@@ -310,16 +309,17 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
       e.len = len;
       e.prob = p;
       e.flags = fl;
-      __threadfence_block();
-      *tq_count = n + 1;
+      st_release(tq_count, n + 1);
     }
     __syncwarp();
   };
-  // wait until tile number n is published (bounded like every wait)
+  // wait until tile number n is published (bounded like every wait).  The count
+  // is released after the tile's slot and descriptor and acquired here by every
+  // lane, so plain reads of both may follow.
   auto published = [&](int n) {
-    if (__all_sync(0xffffffffu, *tq_count > n)) return true;
+    if (__all_sync(0xffffffffu, ld_acquire(tq_count) > n)) return true;
     const long long t0 = clock64();
-    while (__any_sync(0xffffffffu, *tq_count <= n)) {
+    while (__any_sync(0xffffffffu, ld_acquire(tq_count) <= n)) {
       if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_CYCLES)) {
         atomicOr(err, 1u);
         return false;

@@ -120,6 +120,16 @@ __device__ __forceinline__ float fld(const float* __restrict__ p, float s, long 
   return p ? __ldg(p + i) : s;
 }
 
+// A word in shared memory that publishes what the CTA wrote before it.
+__device__ __forceinline__ void st_release(uint32_t addr, int v) {
+  asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(uint32_t addr) {
+  int v;
+  asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 // 4-byte global -> shared copy that completes asynchronously (cp.async);
 // cp_async_wait_all() waits for all of the thread's outstanding copies
 __device__ __forceinline__ void cp_async4(float* sdst, const float* gsrc) {
