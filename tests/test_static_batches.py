@@ -62,3 +62,44 @@ def test_batch_of_many_short_tiles(cuda, storage, dims, shape, dirs, ndir):
     for p, (E, F) in zip(probs, got):
         E1, F1 = _alone(p, storage, 3)
         assert np.array_equal(E, E1) and np.array_equal(F, F1)
+
+
+@pytest.mark.parametrize("storage", [F32, F16, BF16])
+@pytest.mark.parametrize("lam", [0.0, 0.3])
+def test_non_finite_2d_problem_stays_alone(cuda, storage, lam):
+    """A diverged 2D problem of a batch reaches no other one, though its tiles
+    and theirs go through the same CTAs (1024 tiles, one or two CTAs an SM)."""
+    shape = (1, 2048, 66)
+    probs = [dict(dims=2, shape=shape, dirs=RING(120), bc=(P, P, P), fluid=dict(kappa_0=2.0 + k, lam=lam),
+                  state=W.random_populations(120, shape, k)) for k in range(4)]
+    probs[0]["state"][:] = np.inf
+    got, _ = _batch(probs, storage, 2)
+    assert not np.isfinite(got[0][0]).any()
+    for p, (E, F) in list(zip(probs, got))[1:]:
+        E1, F1 = _alone(p, storage, 2)
+        assert np.isfinite(E1).all()
+        assert np.array_equal(E, E1) and np.array_equal(F, F1)
+
+
+@pytest.mark.parametrize("storage", [F32, F16, BF16])
+def test_non_finite_rows_of_a_2d_grid_reach_their_neighbours_only(cuda, storage):
+    """One step moves a value by one row at most, whichever CTA ran which tile."""
+    ny, nx = 640, 1024
+    h = lbrt.lb_rt_create(2, nx, ny, 1, storage=storage, bc=(P, V, P), **RING(120))
+    try:
+        lbrt.lb_rt_set_fluid(h, kappa_0=1.0)
+        E = []
+        for bad in (False, True):
+            E0 = W.random_fields((1, ny, nx), 5, 0.5, 1.5)
+            if bad:
+                E0[0, :ny // 2] = np.inf
+            lbrt.lb_rt_set_state(h, E0, lbrt.LB_RT_STATE_ISOTROPIC)
+            lbrt.lb_rt_step(h, 1)
+            E.append(np.zeros((1, ny, nx), np.float32))
+            lbrt.lb_rt_moments(h, E[-1])
+    finally:
+        lbrt.lb_rt_destroy(h)
+    far = ny // 2 + 1
+    assert np.isfinite(E[0]).all()
+    assert not np.isfinite(E[1][0, :far]).any()
+    assert np.array_equal(E[0][0, far:], E[1][0, far:])
