@@ -76,7 +76,9 @@ __global__ void k_decode(Grid g, int Next, const int* __restrict__ int_of_ext,
 __global__ void k_frozen(Grid g, int Next, const int* __restrict__ int_of_ext, int ncells,
                          const int64_t* __restrict__ cells, const float* __restrict__ vals,
                          float* __restrict__ pop, double* injection) {
-  const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
+  // 32 threads a cell: their number passes 2^32 before ncells passes an int
+  const long long c = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x % 32;
   if (c >= ncells) return;
   int x, y, z;
   site_xyz(g, cells[c], x, y, z);
@@ -369,7 +371,9 @@ __global__ void k_frozen16(Grid g, int Ni, int Next, const int* __restrict__ int
                            const int64_t* __restrict__ cells, const float* __restrict__ vals,
                            ST* __restrict__ pop, float* __restrict__ e, double* injection,
                            DirTable t) {
-  const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
+  // 32 threads a cell: their number passes 2^32 before ncells passes an int
+  const long long c = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x % 32;
   if (c >= ncells) return;
   int x, y, z;
   site_xyz(g, cells[c], x, y, z);
@@ -531,7 +535,7 @@ cudaError_t launch_frozen(const Grid& g, int Ni, int Next, const int* int_of_ext
                           const int64_t* cells, const float* vals, void* pop, float* e,
                           int storage, const DirTable& t, double* injection_acc, cudaStream_t s) {
   if (ncells <= 0) return cudaSuccess;
-  const int nb = (ncells + BLK / 32 - 1) / (BLK / 32);  // a warp per cell
+  const int nb = (int)((ncells + BLK / 32 - 1LL) / (BLK / 32));  // a warp per cell
   if (storage == ST_F32)
     k_frozen<<<nb, BLK, 0, s>>>(g, Next, int_of_ext, ncells, cells, vals,
                                 static_cast<float*>(pop), injection_acc);
