@@ -48,7 +48,8 @@ struct lb_rt {
   double* partials = nullptr;
   int partials_cap = 0;
   double* acc = nullptr;       // 8 doubles, see k_budget_finalize
-  unsigned* err = nullptr;     // device error word, followed by the 2 words of the tile counter
+  unsigned* err = nullptr;     // device error word, the 2 words of the tile counter, blocks done
+                               // of the budget's last kernel
   unsigned* err_host = nullptr;  // page-locked host copy of it, read after each sync
   float* scratch = nullptr;    // moments staging for host outputs [10][sites]
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;

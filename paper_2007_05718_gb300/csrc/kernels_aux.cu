@@ -98,25 +98,54 @@ __global__ void k_frozen(Grid g, int Next, const int* __restrict__ int_of_ext, i
 // acc layout: [0] total, [1] initial, [2] outflow, [3] source, [4] injection,
 // [5] steps, [6] injection of the current step (added by the frozen kernel).
 // partials: [nblocks][2] = (sum E*, sum E_collided) of the step just taken.
-__global__ void k_budget_finalize(const double* __restrict__ partials, int nblocks, double* acc) {
-  __shared__ double sa[BLK], sb[BLK];
-  double a = 0.0, b = 0.0;
-  for (int k = threadIdx.x; k < nblocks; k += blockDim.x) {
-    a += partials[2 * k];
-    b += partials[2 * k + 1];
-  }
-  sa[threadIdx.x] = a;
-  sb[threadIdx.x] = b;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sa[threadIdx.x] += sa[threadIdx.x + w];
-      sb[threadIdx.x] += sb[threadIdx.x + w];
+// A block sums kFinSlots of them; where there are more, every block leaves its
+// sum in its first slot and the last one to finish adds those up in their order
+// (a slot per 32 sites: 17 blocks at 93x61x47, 1024 at 256^3).  The rate of FP64
+// additions (two a cycle and SM) is what counts: hence many blocks, and a tree in
+// shared memory instead of shuffles, which add in every lane.
+constexpr int kFinSlots = 2 * BLK;
+__global__ void k_budget_finalize(double* partials, int nblocks, double* acc, unsigned* done) {
+  __shared__ double2 sh[BLK];
+  __shared__ bool last;
+  double2* const slots = reinterpret_cast<double2*>(partials);
+  // sum of slots k0, k0 + stride .. < k1, in sh[0]
+  auto block_sum = [&](long long k0, long long k1, int stride) {
+    double2 a = make_double2(0.0, 0.0);
+    long long k = k0 + (long long)threadIdx.x * stride;
+    if (k < k1) a = __ldcg(slots + k);
+    while ((k += BLK * stride) < k1) {
+      const double2 v = __ldcg(slots + k);
+      a.x += v.x;
+      a.y += v.y;
+    }
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    for (int w = BLK / 2; w > 0; w >>= 1) {
+      if (threadIdx.x < w) {
+        sh[threadIdx.x].x += sh[threadIdx.x + w].x;
+        sh[threadIdx.x].y += sh[threadIdx.x + w].y;
+      }
+      __syncthreads();
+    }
+  };
+  const long long first = (long long)blockIdx.x * kFinSlots;
+  block_sum(first, min((long long)nblocks, first + kFinSlots), 1);
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) {
+      __stcg(slots + first, sh[0]);
+      __threadfence();
+      last = atomicAdd(done, 1u) == gridDim.x - 1;
+      if (last) {
+        *done = 0;
+        __threadfence();
+      }
     }
     __syncthreads();
+    if (!last) return;
+    block_sum(0, (long long)gridDim.x * kFinSlots, kFinSlots);
   }
   if (threadIdx.x == 0) {
-    const double estar = sa[0], ecoll = sb[0];
+    const double estar = sh[0].x, ecoll = sh[0].y;
     const double inj = acc[6];
     acc[2] += acc[0] - estar;   // outflow through vacuum faces
     acc[3] += ecoll - estar;    // collision source
@@ -564,9 +593,10 @@ cudaError_t launch_coupling(const Grid& g, int N, const void* pop, const float* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_budget_finalize(const double* partials, int nblocks, double* acc,
+cudaError_t launch_budget_finalize(double* partials, int nblocks, double* acc, unsigned* done,
                                    cudaStream_t s) {
-  k_budget_finalize<<<1, BLK, 0, s>>>(partials, nblocks, acc);
+  const int blocks = std::max(1, (int)((nblocks + (long long)kFinSlots - 1) / kFinSlots));
+  k_budget_finalize<<<blocks, BLK, 0, s>>>(partials, nblocks, acc, done);
   return cudaGetLastError();
 }
 

@@ -128,7 +128,7 @@ struct TileInfo {
 
 // Shared memory (bytes), every offset known at compile time (GM = the plan's
 // largest warp count; run-time offsets were recomputed all over the loop):
-// TMA barriers [GM][2] | E barriers [3] | P, C | tile queue | budget [GM][2] f64 | coef
+// TMA barriers [GM][2] | E barriers [3] | P, C | tile queue | coef
 // [2][ZC][NC][64] f32 | site fields of two batches [2][2 ZC][3 or 4][32] f32 |
 // descriptors of 4 tiles (batch) | E ring [3][ESLOT] | partials [GM][ZC][1 or 4][64] f32 |
 // directions [GM DPT] | ring [G][2][SLOT]
@@ -138,8 +138,7 @@ struct StLayout {
   static constexpr int PBAR = EBAR + 8 * kEring;
   static constexpr int CBAR = PBAR + 8;
   static constexpr int TILEQ = CBAR + 8;  // 4 TileInfo, the count published
-  static constexpr int BSUM = TILEQ + 4 * (int)sizeof(TileInfo) + 8;
-  static constexpr int COEF = (BSUM + 16 * GM + 127) / 128 * 128;
+  static constexpr int COEF = (TILEQ + 4 * (int)sizeof(TileInfo) + 4 + 127) / 128 * 128;
   static constexpr int FIELDS = COEF + 2 * ZC * (FLUX ? 5 : 2) * 256;
   static constexpr int DESC = FIELDS + 2 * (2 * ZC) * (FLUX ? 4 : 3) * 128;
   static constexpr int ERING = (DESC + (BATCH ? 4 * (int)sizeof(ProblemDesc) : 0) + 127) / 128 * 128;
@@ -169,7 +168,10 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
                                             const int G) {
   constexpr bool F32 = SV<ST>::F32;
   constexpr bool BATCH = MODE == 1;
-  constexpr bool MOM = MODE == 2;
+  constexpr bool MOM = (MODE & 3) == 2;
+  // the energy budget has kernels of its own: tested at run time it cost the
+  // step without it 1 % (256^3 x 162 float32, 4.74 against 4.78 ms)
+  constexpr bool BUDGET = MODE & 4;
   static_assert(!MOM || (FLUX && F32), "the moments epilogue needs the flux and float32 storage");
   constexpr int BOX = SV<ST>::BOX;
   constexpr int SLOT = st_slot_bytes<ST, DPT, ZC>();
@@ -187,7 +189,6 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
   float* const part = reinterpret_cast<float*>(smem_raw + L::PART);
   float* const coef = reinterpret_cast<float*>(smem_raw + L::COEF);
   DirC<FLUX>* const dirs = reinterpret_cast<DirC<FLUX>*>(smem_raw + L::DIRS);
-  double* const bsum = reinterpret_cast<double*>(smem_raw + L::BSUM);
   const uint32_t e_bar = smem0 + L::EBAR, p_bar = smem0 + L::PBAR, c_bar = smem0 + L::CBAR;
 
   const int i0 = g * DPT;
@@ -214,7 +215,6 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
   }
   if (lane == 0) {
     for (int r = 0; r < kRing; ++r) mbar_init(smem0 + 8 * (g * kRing + r), 1);
-    bsum[2 * g] = bsum[2 * g + 1] = 0.0;
     if (g == 0) {
       for (int r = 0; r < kEring; ++r) mbar_init(e_bar + 8 * r, 1);
       mbar_init(p_bar, G);
@@ -262,8 +262,8 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
   // row finds it in L2.  (With tiles dealt out in advance CTAs drift apart, and
   // on some boards the upwind rows came from DRAM a second time: the 256^3 x
   // 162 float32 step took 8.0 ms there against 5.3 ms.)  Which CTA runs a tile
-  // does not change its arithmetic.  sched == nullptr (the energy budget keeps
-  // per-CTA partial sums, whose order is fixed): tiles cta, cta + ncta, ...
+  // does not change its arithmetic, nor the energy budget, which has a partial
+  // sum per unit.
   // Warp 0 takes tile n + 1 when it opens tile n and publishes its geometry in
   // the queue (slot n + 1 mod 4) while it works on the tile's first item.
   volatile TileInfo* const tq = reinterpret_cast<volatile TileInfo*>(smem_raw + L::TILEQ);
@@ -328,7 +328,6 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     return true;
   };
   auto items_of = [&](int len) { return len < 0 ? -len : tile_items<ZC>(len); };
-  long long my_tile = cta;  // warp 0: the tile taken last
   unsigned grabbed = 0;     // warp 0, lane 0: counter value of the tile to publish
   bool to_publish = false;
 
@@ -342,8 +341,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     // behind the stores in flight
     if (!to_publish || (m < 2 && m + kRing + 1 < M)) return;
     to_publish = false;
-    my_tile = sched ? (long long)ncta + __shfl_sync(0xffffffffu, grabbed, 0) : my_tile + ncta;
-    publish(tn + 1, my_tile);
+    publish(tn + 1, (long long)ncta + __shfl_sync(0xffffffffu, grabbed, 0));
   };
   auto open_tile = [&]() {  // false: no tile left
     ++tn;
@@ -366,6 +364,8 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     t_base = static_cast<ST*>(D.out) + (long long)i0 * D.g.si + (long long)t_z * D.g.sz +
              (long long)(t_y + 1) * D.g.sy + (t_x0 + 2 * lane + GL);
     if (g == 0) {
+      // (sched is never null; without the test the compiler merges this branch
+      // with others and spills up to 186 bytes: 128^3 x 42 took 2.4 times as long)
       if (sched && lane == 0) grabbed = atomicAdd(sched, 1u);
       to_publish = true;
     }
@@ -508,16 +508,15 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
       }
     }
     arrive(c_bar);
-    if (!BATCH && D.budget_partials) {
-      double a = v ? (double)E : 0.0, b = v ? (double)cc.Enew : 0.0;
-      for (int s = 16; s > 0; s >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, s);
-        b += __shfl_xor_sync(0xffffffffu, b, s);
-      }
-      if (lane == 0) {
-        bsum[2 * g] += a;
-        bsum[2 * g + 1] += b;
-      }
+    if constexpr (BUDGET) {
+      // Sums over the 32 sites in FP64, whose additions are slow here (two a
+      // cycle and SM): lanes 0 - 15 go on with E*, lanes 16 - 31 with E'.
+      const double a = v ? (double)E : 0.0, b = v ? (double)cc.Enew : 0.0;
+      double r = (lane < 16 ? a : b) + __shfl_xor_sync(0xffffffffu, lane < 16 ? b : a, 16);
+      for (int s = 8; s > 0; s >>= 1) r += __shfl_xor_sync(0xffffffffu, r, s);
+      const int x32 = tq[c.flags >> 24].x0 + ((u & 1) << 5);
+      if (!(lane & 15) && x32 < gr.nx && (c.flags >> (8 + j) & 1))
+        one.budget_partials[2 * (((long long)z * gr.ny + y) * ((gr.nx + 31) / 32) + x32 / 32) + lane / 16] = r;
     }
     if (v) {
       if constexpr (MOM) {
@@ -889,7 +888,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     }
   }
   // the last CTA to leave puts the tile counter back
-  if (sched && g == 0 && lane == 0 && atomicAdd(sched + 1, 1u) == (unsigned)ncta - 1) {
+  if (g == 0 && lane == 0 && atomicAdd(sched + 1, 1u) == (unsigned)ncta - 1) {
     sched[0] = 0;
     sched[1] = 0;
   }
@@ -901,18 +900,6 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     if (g == 0)
       for (int qq = waited; qq < issued; ++qq)
         mbar_wait(e_bar + 8 * (qq % kEring), (uint32_t)((qq / kEring) & 1), err);
-  }
-  if (!BATCH && one.budget_partials) {
-    cta_sync<PART>(32 * G);
-    if (g == 0 && lane == 0) {
-      double a = 0.0, b = 0.0;
-      for (int w = 0; w < G; ++w) {
-        a += bsum[2 * w];
-        b += bsum[2 * w + 1];
-      }
-      atomicAdd(one.budget_partials + 2 * cta, a);
-      atomicAdd(one.budget_partials + 2 * cta + 1, b);
-    }
   }
 }
 

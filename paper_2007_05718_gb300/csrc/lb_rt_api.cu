@@ -249,7 +249,8 @@ lb_rt_status run_steps(lb_rt* h, int nsteps, float* mE, float* mF) {
     int nblocks = 0;
     if (h->cfg.budget) {
       L.budget_partials = h->partials;
-      CK(h, cudaMemsetAsync(h->partials, 0, sizeof(double) * 2 * h->partials_cap, h->stream));
+      if (h->cfg.moving)
+        CK(h, cudaMemsetAsync(h->partials, 0, sizeof(double) * 2 * h->partials_cap, h->stream));
     }
     cudaError_t e = h->cfg.moving
                         ? launch_step_moving(L, h->mc, h->table, h->cfg.storage, h->stream, &nblocks)
@@ -263,7 +264,7 @@ lb_rt_status run_steps(lb_rt* h, int nsteps, float* mE, float* mF) {
       if (e != cudaSuccess) return cuda_fail(h, e, "frozen kernel");
     }
     if (h->cfg.budget) {
-      e = launch_budget_finalize(h->partials, nblocks, h->acc, h->stream);
+      e = launch_budget_finalize(h->partials, nblocks, h->acc, h->err + 3, h->stream);
       if (e != cudaSuccess) return cuda_fail(h, e, "budget kernel");
     }
     h->cur ^= 1;
@@ -412,14 +413,14 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
     alloc((void**)&h->ef[0], h->ef_bytes);
     alloc((void**)&h->ef[1], h->ef_bytes);
   }
-  // budget partials: one slot pair per CTA of the step kernel; every step
-  // kernel's grid is at most ceil(nx/32) x ny x nz CTAs
+  // budget partials: one slot pair per 32 sites of a row (static step), which is
+  // at least one per CTA of the moving step
   const long long step_blocks = (long long)((cfg->nx + 31) / 32) * cfg->ny * cfg->nz;
   h->partials_cap = (int)std::max<long long>(max_blocks, step_blocks);
   alloc((void**)&h->partials, sizeof(double) * 2 * h->partials_cap);
   alloc((void**)&h->acc, sizeof(double) * 8);
   alloc((void**)&h->d_int_of_ext, sizeof(int) * h->N);
-  alloc((void**)&h->err, 3 * sizeof(unsigned));
+  alloc((void**)&h->err, 4 * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->err_host, sizeof(unsigned), cudaHostAllocDefault);
   if (e != cudaSuccess) {
     g_create_msg = std::string("allocation: ") + cudaGetErrorString(e);
@@ -437,7 +438,7 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->d_int_of_ext, h->int_of_ext.data(), sizeof(int) * h->N,
                         cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, 3 * sizeof(unsigned), h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, 4 * sizeof(unsigned), h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     g_create_msg = std::string("init: ") + cudaGetErrorString(e);

@@ -93,8 +93,9 @@ struct StepLaunch {
   const CUtensorMap* tmap_e;   // 16-bit storage: TMA descriptor of the E array at t
   const float* e_in;           // 16-bit storage: E array at t (padded, float32)
   float* e_out;                // 16-bit storage: E array at t + dt (padded, float32)
-  double* budget_partials;  // [nblocks][2] (sum E*, sum E_collided) or nullptr
-  long long partials_cap;   // slots available; a launcher whose grid is larger refuses
+  double* budget_partials;  // [nblocks][2] (sum E*, sum E_collided) or nullptr; a slot per 32
+                            // sites of a row (static: stored) or CTA (moving: added to zeros)
+  long long partials_cap;   // slots available; a launcher that needs more refuses
   unsigned* err;            // device error word
   unsigned* sched;          // static step: tile counter, CTAs done (2 words, zero between launches)
   float* mom_E;             // FP32 static step: E of the new state, dense [sites], or nullptr
@@ -167,7 +168,7 @@ cudaError_t launch_decode(const Grid& g, int Next, const int* int_of_ext, const 
 cudaError_t launch_frozen(const Grid& g, int Ni, int Next, const int* int_of_ext, int ncells,
                           const int64_t* cells, const float* vals, void* pop, float* e,
                           int storage, const DirTable& t, double* injection_acc, cudaStream_t s);
-cudaError_t launch_budget_finalize(const double* partials, int nblocks, double* acc,
+cudaError_t launch_budget_finalize(double* partials, int nblocks, double* acc, unsigned* done,
                                    cudaStream_t s);
 // Coupling outputs J [sites], H [3][sites], S [4][sites] (any may be null).
 cudaError_t launch_coupling(const Grid& g, int N, const void* pop, const float* e, int storage,

@@ -96,6 +96,7 @@ cudaError_t launch_step_static(const StepLaunch& L, const StaticCoef& c, const D
   StaticCall k;
   k.mode = one.mom_E || one.mom_F ? 2 : 0;
   k.flux = has_flux(c);
+  k.budget = L.budget_partials != nullptr;
   k.dpt = L.dpt;
   k.zc = L.zc;
   k.N = L.N;
@@ -107,12 +108,13 @@ cudaError_t launch_step_static(const StepLaunch& L, const StaticCoef& c, const D
   if (fl) k.ctas = L.ctas_flux, one.nzc = L.nzc_flux, one.ntiles = k.ntiles = static_tiles(L.g, L.nzc_flux);
   k.one = &one;
   k.nprob = 1;
-  if (L.budget_partials && k.ctas > L.partials_cap) return cudaErrorInvalidValue;
-  if (nblocks) *nblocks = k.ctas;
+  // energy budget: a partial sum per 32 sites of a row, stored by the unit that
+  // owns them, so that its order does not depend on who ran which tile
+  const long long nslots = (long long)((L.g.nx + 31) / 32) * L.g.ny * L.g.nz;
+  if (L.budget_partials && nslots > L.partials_cap) return cudaErrorInvalidValue;
+  if (nblocks) *nblocks = (int)nslots;
   k.err = L.err;
-  // the budget's per-CTA partial sums want a fixed assignment of tiles to CTAs;
-  // otherwise the counter (256^3 x 162 float32: 9.2 ms dealt out, 5.7 counted)
-  k.sched = L.budget_partials ? nullptr : L.sched;
+  k.sched = L.sched;
   k.dirs = &t;
   k.stream = s;
   return run(storage, k);

@@ -19,6 +19,7 @@ constexpr size_t kStaticSmemMax = 226 * 1024;
 
 struct StaticCall {
   int mode = 0;              // 0 one problem, 1 batch, 2 one problem with the E, F epilogue
+  bool budget = false;       // modes 0 and 2: with the energy budget
   bool flux = false;         // some problem has lambda != 0 (or the epilogue needs F)
   bool alt = false;          // batch: the alternative kernel of the plan
   int dpt = 0, zc = 0, N = 0;  // directions per warp, planes per batch, internal directions
@@ -28,7 +29,7 @@ struct StaticCall {
   const ProblemDesc* table = nullptr;  // batch: device array
   int nprob = 0, ntiles = 0, ctas = 0;
   unsigned* err = nullptr;
-  unsigned* sched = nullptr; // tile counter and CTAs done (zero between launches), or null
+  unsigned* sched = nullptr; // tile counter and CTAs done (zero between launches)
   const DirTable* dirs = nullptr;
   cudaStream_t stream = nullptr;
   int* per_sm = nullptr;     // set: only query the resident CTAs per SM

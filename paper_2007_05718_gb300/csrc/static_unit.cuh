@@ -44,8 +44,13 @@ cudaError_t static_plan(const StaticCall& c) {
     return c.flux ? static_kernel<ST, 1, true, DPT, ZC, HU, H, MAXT, REGS>(c)
                   : static_kernel<ST, 1, false, DPT, ZC, HU, H, MAXT, REGS>(c);
   if constexpr (SV<ST>::F32) {
-    if (c.mode == 2) return static_kernel<ST, 2, true, DPT, ZC, HU, H, MAXT, REGS>(c);
+    if (c.mode == 2)
+      return c.budget ? static_kernel<ST, 2 + 4, true, DPT, ZC, HU, H, MAXT, REGS>(c)
+                      : static_kernel<ST, 2, true, DPT, ZC, HU, H, MAXT, REGS>(c);
   }
+  if (c.budget)
+    return c.flux ? static_kernel<ST, 4, true, DPT, ZC, HU, H, MAXT, REGS>(c)
+                  : static_kernel<ST, 4, false, DPT, ZC, HU, H, MAXT, REGS>(c);
   return c.flux ? static_kernel<ST, 0, true, DPT, ZC, HU, H, MAXT, REGS>(c)
                 : static_kernel<ST, 0, false, DPT, ZC, HU, H, MAXT, REGS>(c);
 }
