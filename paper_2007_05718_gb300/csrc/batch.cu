@@ -34,7 +34,8 @@ struct Member {
 struct Group {
   DirTable table{};
   int Ni = 0, dpt = 0, zc = 0;
-  int per_sm = 0;         // resident CTAs per SM of the batched kernel
+  // resident CTAs per SM of the batched kernels: [alternative kernel][flux terms]
+  int per_sm[2][2] = {{0, 0}, {0, 0}};
   int zchunk = 16;        // planes per tile
   // autotuner: candidates are timed on successive ticks of a new member set
   std::vector<int> cands;
@@ -46,9 +47,9 @@ struct Group {
   int ctas = 0;           // CTAs of the last launch
   bool paired = false;    // the last tick ran the group in a launch shared with another group
   // alternative batched kernel of the same layout (batch_alt_zc): its planes
-  // per batch (0: none) and residency; alt = 1 while it is in use.  The
+  // per batch (0: none); alt = 1 while it is in use.  The
   // autotuner times it at the best z chunk after the z-chunk candidates.
-  int alt_zc = 0, alt_per_sm = 0, alt = 0;
+  int alt_zc = 0, alt = 0;
   int stage = 0;          // tuning: 0 z chunks, 1 the alternative kernel
   int zc_now() const { return alt ? alt_zc : zc; }
   int last_zc = 0;        // planes per batch of the kernel of the last launch
@@ -96,7 +97,7 @@ struct lb_rt_batch {
   // resident CTAs per SM of the paired kernel, and the autotuner's choice
   // (mode 2): -1 undecided, 0 separate launches, 1 paired launch, timed on
   // one tick each and normalised per site-direction update
-  int pair_a = -1, pair_b = -1, pair_per_sm = 0;
+  int pair_a = -1, pair_b = -1, pair_per_sm[2] = {0, 0};  // [flux terms]
   int pair_choice = -1, pair_trial = 0;
   long long pair_sites = 0;  // sites of the two groups when the choice was timed
   double pair_cost[2] = {0.0, 0.0};
@@ -296,8 +297,15 @@ lb_rt_status lb_rt_batch_admit(lb_rt_batch* b, const lb_rt_config* cfg, const lb
     g.Ni = h->Ni;
     g.dpt = h->dpt;
     g.zc = h->zc;
-    cudaError_t e = occupancy_static_batch(c.storage, g.dpt, g.zc, g.Ni, &g.per_sm);
-    if (e == cudaSuccess && g.per_sm < 1) e = cudaErrorInvalidConfiguration;
+    auto query = [&](int alt) {
+      cudaError_t e = cudaSuccess;
+      for (int flux = 0; flux < 2 && e == cudaSuccess; ++flux) {
+        e = occupancy_static_batch(c.storage, g.dpt, g.zc, g.Ni, alt, flux, &g.per_sm[alt][flux]);
+        if (e == cudaSuccess && g.per_sm[alt][flux] < 1) e = cudaErrorInvalidConfiguration;
+      }
+      return e;
+    };
+    cudaError_t e = query(0);
     if (e == cudaSuccess) e = cudaEventCreate(&g.ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&g.ev1);
     if (e != cudaSuccess) {
@@ -308,9 +316,7 @@ lb_rt_status lb_rt_batch_admit(lb_rt_batch* b, const lb_rt_config* cfg, const lb
     for (int z : kZCandidates) g.cands.push_back(z);
     g.cost.assign(g.cands.size() + 1, 0.0);  // z chunks, then the alternative kernel
     g.alt_zc = batch_alt_zc(g.dpt, g.zc);
-    if (g.alt_zc &&
-        (occupancy_static_batch(c.storage, g.dpt, g.zc, g.Ni, &g.alt_per_sm, 1) != cudaSuccess ||
-         g.alt_per_sm < 1)) {
+    if (g.alt_zc && query(1) != cudaSuccess) {
       (void)cudaGetLastError();
       g.alt_zc = 0;
     }
@@ -452,17 +458,21 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
   if (pa >= 0 && (pa != b->pair_a || pb != b->pair_b)) {
     const Group& A = b->groups[pa];
     const Group& B = b->groups[pb];
-    int per_sm = 0;
-    cudaError_t e = occupancy_static_batch_pair(b->cfg.storage, A.dpt, A.zc_now(), A.Ni, B.dpt,
-                                                B.zc_now(), B.Ni, &per_sm);
-    if (e != cudaSuccess) return bcuda(b, e, "paired kernel occupancy");
+    int per_sm[2] = {0, 0};
+    for (int flux = 0; flux < 2; ++flux) {
+      cudaError_t e = occupancy_static_batch_pair(b->cfg.storage, A.dpt, A.zc_now(), A.Ni, B.dpt,
+                                                  B.zc_now(), B.Ni, flux, &per_sm[flux]);
+      if (e != cudaSuccess) return bcuda(b, e, "paired kernel occupancy");
+    }
     b->pair_a = pa;
     b->pair_b = pb;
-    b->pair_per_sm = per_sm;
+    b->pair_per_sm[0] = per_sm[0];
+    b->pair_per_sm[1] = per_sm[1];
     b->pair_choice = -1;
     b->pair_trial = 0;
   }
-  if (pa >= 0 && b->pair_per_sm < 1) pa = pb = -1;
+  const int pair_per_sm = pa >= 0 ? b->pair_per_sm[group_flux[pa] || group_flux[pb]] : 0;
+  if (pair_per_sm < 1) pa = pb = -1;
   bool pair_timed = false;  // this tick is one of mode 2's two trials
   if (pa >= 0 && b->cfg.pair_groups == 2) {
     // timed again when the pair's sites have changed by more than 2x
@@ -560,7 +570,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       const Launch& Bl = L0.group == pa ? L1 : L0;
       const Group& GA = b->groups[pa];
       const Group& GB = b->groups[pb];
-      long long S = std::min<long long>((long long)b->pair_per_sm * b->sms,
+      long long S = std::min<long long>((long long)pair_per_sm * b->sms,
                                         (long long)A.ntiles + Bl.ntiles);
       if (S >= 2) {
         const double wa = (double)A.sd / (GA.Ni / GA.dpt), wb = (double)Bl.sd / (GB.Ni / GB.dpt);
@@ -582,7 +592,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     }
     for (size_t i = first_of_step; i < launches.size(); ++i) {
       const Launch& L = launches[i];
-      for (long long v : {(long long)L.group, (long long)group_maps[L.group],
+      for (long long v : {(long long)L.group, (long long)group_maps[L.group], (long long)b->groups[L.group].alt,
                           (long long)L.first, (long long)L.nprob,
                           (long long)L.ntiles, (long long)L.flux, (long long)L.b_group,
                           (long long)L.b_first, (long long)L.b_nprob, (long long)L.b_ntiles,
@@ -627,7 +637,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     };
     auto single = [&](const Launch& L) -> cudaError_t {
       Group& gr = b->groups[L.group];
-      const int per_sm = gr.alt ? gr.alt_per_sm : gr.per_sm;
+      const int per_sm = gr.per_sm[gr.alt][L.flux];
       const int ctas = (int)std::min<long long>((long long)per_sm * b->sms, L.ntiles);
       gr.last_zc = gr.zc_now();
       gr.ctas = ctas;

@@ -232,9 +232,9 @@ lb_rt_status run_steps(lb_rt* h, int nsteps, float* mE, float* mF) {
     if (!h->cfg.moving && h->zc != static_flux_zc(h->dpt)) {
       L.tmap_flux = &h->tmap_flux[h->cur];
       L.tmap_e_flux = h->ef[0] ? &h->emap_flux[h->cur] : nullptr;
-      L.nzc_flux = h->nzc_flux;
-      L.ctas_flux = h->ctas_flux;
     }
+    L.nzc_flux = h->nzc_flux;
+    L.ctas_flux = h->ctas_flux;
     L.tmap_e = h->ef[0] && h->tmap_ok ? &h->emap[h->cur] : nullptr;
     L.e_in = h->ef[h->cur];
     L.e_out = h->ef[h->cur ^ 1];
@@ -466,10 +466,10 @@ lb_rt_status lb_rt_create(const lb_rt_config* cfg, lb_rt** out) {
     }
     h->tmap_ok = true;
     e = plan_static_grid(h->grid, h->Ni, h->dpt, h->zc, cfg->storage, &h->nzc, &h->ctas,
-                         cfg->moving != 0);
-    if (e == cudaSuccess && !cfg->moving && h->zc != static_flux_zc(h->dpt))
+                         cfg->moving != 0, false);
+    if (e == cudaSuccess && !cfg->moving)
       e = plan_static_grid(h->grid, h->Ni, h->dpt, static_flux_zc(h->dpt), cfg->storage, &h->nzc_flux,
-                           &h->ctas_flux);
+                           &h->ctas_flux, false, true);
     if (e != cudaSuccess) {
       g_create_msg = std::string("static kernel grid: ") + cudaGetErrorString(e);
       lb_rt_destroy(h);

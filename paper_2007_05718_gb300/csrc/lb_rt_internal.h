@@ -86,7 +86,7 @@ struct StepLaunch {
   const void* in;      // populations at t (padded layout)
   void* out;           // populations at t + dt
   const CUtensorMap* tmap_in;  // TMA descriptor of `in` (host copy)
-  // flux terms, where their boxes (static_flux_zc planes) differ, or null
+  // flux terms: maps where their boxes (static_flux_zc planes) differ, or null; grid
   const CUtensorMap* tmap_flux;
   const CUtensorMap* tmap_e_flux;
   int nzc_flux, ctas_flux;
@@ -136,7 +136,7 @@ struct BatchLaunch {
   unsigned* err;
 };
 cudaError_t launch_static_batch(const BatchLaunch& B, const DirTable& t, cudaStream_t s);
-cudaError_t occupancy_static_batch(int storage, int dpt, int zc, int Ni, int* per_sm, int alt = 0);
+cudaError_t occupancy_static_batch(int storage, int dpt, int zc, int Ni, int alt, bool flux, int* per_sm);
 int batch_alt_zc(int dpt, int zc);
 // Two groups with different tile plans in ONE batched launch: group A's
 // problems run on CTAs 0 .. ctas_a - 1 of the ctas-CTA grid, group B's on the
@@ -146,7 +146,7 @@ bool static_batch_pair_supported(int dpt_a, int zc_a, int dpt_b, int zc_b);
 cudaError_t launch_static_batch_pair(const BatchLaunch& A, const DirTable& ta, const BatchLaunch& B,
                                      const DirTable& tb, int ctas_a, int ctas, cudaStream_t s);
 cudaError_t occupancy_static_batch_pair(int storage, int dpt_a, int zc_a, int Na, int dpt_b,
-                                        int zc_b, int Nb, int* per_sm);
+                                        int zc_b, int Nb, bool flux, int* per_sm);
 
 // Kernel launchers.  Return cudaGetLastError() (or an error without
 // launching when the configuration is not supported).
@@ -191,11 +191,11 @@ struct TilePlan {
 int static_plan_lists(int storage, const TilePlan* lists[2], int counts[2]);
 int static_zc(int dpt, const Grid& g);  // planes per batch
 int static_flux_zc(int dpt);            // the same with the flux terms
-cudaError_t occupancy_static(int storage, int dpt, int zc, int Ni, int* per_sm);
+cudaError_t occupancy_static(int storage, int dpt, int zc, int Ni, bool flux, int* per_sm);
 // z chunks and CTA count of the tiled kernels' persistent grid for this
 // grid and plan on the current device (occupancy query).
 cudaError_t plan_static_grid(const Grid& g, int Ni, int dpt, int zc, int storage, int* nzc,
-                             int* ctas, bool moving = false);
+                             int* ctas, bool moving, bool flux);
 // Moving fluid, FP32 populations, TMA tiles (kernels_tma_moving.cu): one
 // plane per batch; plans (directions per warp, 1, thread cap).
 extern const int kTilePlansMoving[][3];

@@ -78,7 +78,8 @@ cudaError_t run_pair(int storage, const StaticPairCall& c) {
 cudaError_t launch_step_static(const StepLaunch& L, const StaticCoef& c, const DirTable& t, int storage,
                                cudaStream_t s, int* nblocks) {
   const bool f32 = storage == ST_F32;
-  if (!L.tmap_in || (!f32 && (!L.tmap_e || !L.e_out)) || L.nzc < 1 || L.nzc > march_length(L.g) || L.ctas < 1)
+  if (!L.tmap_in || (!f32 && (!L.tmap_e || !L.e_out)) || L.nzc < 1 || L.nzc > march_length(L.g) || L.ctas < 1 ||
+      L.nzc_flux < 1 || L.nzc_flux > march_length(L.g) || L.ctas_flux < 1)
     return cudaErrorInvalidValue;
   ProblemDesc one{};
   one.g = L.g;
@@ -102,9 +103,9 @@ cudaError_t launch_step_static(const StepLaunch& L, const StaticCoef& c, const D
   k.N = L.N;
   k.ntiles = one.ntiles;
   k.ctas = L.ctas;
-  const bool fl = (k.flux || k.mode == 2) && L.tmap_flux;
-  k.tmap = fl ? L.tmap_flux : L.tmap_in;
-  k.emap = fl ? L.tmap_e_flux : L.tmap_e;
+  const bool fl = k.flux || k.mode == 2;
+  k.tmap = fl && L.tmap_flux ? L.tmap_flux : L.tmap_in;
+  k.emap = fl && L.tmap_flux ? L.tmap_e_flux : L.tmap_e;
   if (fl) k.ctas = L.ctas_flux, one.nzc = L.nzc_flux, one.ntiles = k.ntiles = static_tiles(L.g, L.nzc_flux);
   k.one = &one;
   k.nprob = 1;
@@ -140,33 +141,27 @@ cudaError_t launch_static_batch(const BatchLaunch& B, const DirTable& t, cudaStr
   return run(B.storage, k);
 }
 
-// resident CTAs per SM, the smaller of the kernels with and without the flux terms
-static cudaError_t occupancy(int storage, int mode, int dpt, int zc, int Ni, int alt, int* per_sm) {
-  int best = 1 << 30;
-  for (int flux = 0; flux < 2; ++flux) {
-    int n = 0;
-    StaticCall k;
-    k.mode = mode;
-    k.flux = flux;
-    k.alt = alt;
-    k.dpt = dpt;
-    k.zc = zc;
-    k.N = Ni;
-    k.per_sm = &n;
-    const cudaError_t e = run(storage, k);
-    if (e != cudaSuccess) return e;
-    best = std::min(best, n);
-  }
-  *per_sm = best;
-  return cudaSuccess;
+// Resident CTAs per SM of the kernel that such a launch takes.  The kernels with
+// and without the flux terms, and the alternative one of a plan, differ: 45
+// float32 directions in a batch are 2, 2 and 3 CTAs of 9 warps.
+static cudaError_t occupancy(int storage, int mode, int dpt, int zc, int Ni, int alt, bool flux, int* per_sm) {
+  StaticCall k;
+  k.mode = mode;
+  k.flux = flux;
+  k.alt = alt;
+  k.dpt = dpt;
+  k.zc = zc;
+  k.N = Ni;
+  k.per_sm = per_sm;
+  return run(storage, k);
 }
 
-cudaError_t occupancy_static(int storage, int dpt, int zc, int Ni, int* per_sm) {
-  return occupancy(storage, 0, dpt, zc, Ni, 0, per_sm);
+cudaError_t occupancy_static(int storage, int dpt, int zc, int Ni, bool flux, int* per_sm) {
+  return occupancy(storage, 0, dpt, zc, Ni, 0, flux, per_sm);
 }
 
-cudaError_t occupancy_static_batch(int storage, int dpt, int zc, int Ni, int* per_sm, int alt) {
-  return occupancy(storage, 1, dpt, zc, Ni, alt, per_sm);
+cudaError_t occupancy_static_batch(int storage, int dpt, int zc, int Ni, int alt, bool flux, int* per_sm) {
+  return occupancy(storage, 1, dpt, zc, Ni, alt, flux, per_sm);
 }
 
 bool static_batch_pair_supported(int dpt_a, int zc_a, int dpt_b, int zc_b) {
@@ -190,24 +185,16 @@ cudaError_t launch_static_batch_pair(const BatchLaunch& A, const DirTable& ta, c
 }
 
 cudaError_t occupancy_static_batch_pair(int storage, int dpt_a, int zc_a, int Na, int dpt_b, int zc_b, int Nb,
-                                        int* per_sm) {
+                                        bool flux, int* per_sm) {
   if (!static_batch_pair_supported(dpt_a, zc_a, dpt_b, zc_b)) return cudaErrorInvalidValue;
-  int best = 1 << 30;
-  for (int flux = 0; flux < 2; ++flux) {
-    int n = 0;
-    StaticPairCall k;
-    k.flux = flux;
-    k.a.N = Na;
-    k.b.N = Nb;
-    static const DirTable no_dirs{};
-    k.dirs_a = k.dirs_b = &no_dirs;
-    k.per_sm = &n;
-    const cudaError_t e = run_pair(storage, k);
-    if (e != cudaSuccess) return e;
-    best = std::min(best, n);
-  }
-  *per_sm = best;
-  return cudaSuccess;
+  static const DirTable no_dirs{};
+  StaticPairCall k;
+  k.flux = flux;
+  k.a.N = Na;
+  k.b.N = Nb;
+  k.dirs_a = k.dirs_b = &no_dirs;
+  k.per_sm = per_sm;
+  return run_pair(storage, k);
 }
 
 // Persistent grid of the tiled kernels: CTAs = resident CTAs per SM x SMs (at
@@ -221,7 +208,7 @@ cudaError_t occupancy_static_batch_pair(int storage, int dpt_a, int zc_a, int Na
 // Moving step: tiles cta, cta + ncta, ...; the count minimises the busiest
 // CTA's share of plane loads.
 cudaError_t plan_static_grid(const Grid& g, int Ni, int dpt, int zc, int storage, int* nzc,
-                             int* ctas, bool moving) {
+                             int* ctas, bool moving, bool flux) {
   const int G = Ni / dpt;
   int per_sm = 0;
   cudaError_t e = cudaErrorInvalidValue;
@@ -229,7 +216,7 @@ cudaError_t plan_static_grid(const Grid& g, int Ni, int dpt, int zc, int storage
     e = storage == ST_F32 ? occupancy_tma_moving(dpt, G, &per_sm)
                           : occupancy_tma16_moving(storage, dpt, G, &per_sm);
   } else {
-    e = occupancy_static(storage, dpt, zc, Ni, &per_sm);
+    e = occupancy_static(storage, dpt, zc, Ni, flux, &per_sm);
   }
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;

@@ -103,3 +103,24 @@ def test_non_finite_rows_of_a_2d_grid_reach_their_neighbours_only(cuda, storage)
     assert np.isfinite(E[0]).all()
     assert not np.isfinite(E[1][0, :far]).any()
     assert np.array_equal(E[0][0, far:], E[1][0, far:])
+
+
+def test_every_batched_kernel_gets_its_own_residency(cuda):
+    """42 float32 directions: the autotuner times the alternative kernel (one
+    plane a batch, 72 registers, three CTAs of nine warps an SM) on its fifth
+    tick, and with more CTAs than the plan's own kernel (two of 96 registers)."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shape = (64, 256, 64)  # 512 tiles or more, whatever the z chunk
+    b = lbrt.lb_rt_batch_create(max_problems=2, storage=F32, steps_per_tick=1)
+    try:
+        s = [lbrt.lb_rt_batch_admit(b, dict(dims=3, nx=64, ny=256, nz=64, **ICO[1]), dict(kappa_0=2.0),
+                                    W.random_fields(shape, k), lbrt.LB_RT_STATE_ISOTROPIC, 100) for k in range(2)]
+        seen = []
+        for _ in range(5):
+            lbrt.lb_rt_batch_tick(b)
+            seen.append((lbrt.lb_rt_batch_plan(b, s[0])[1], lbrt.lb_rt_batch_tuning(b, s[0])[1]))
+        lbrt.lb_rt_batch_sync(b)
+    finally:
+        lbrt.lb_rt_batch_destroy(b)
+    assert seen == [(2, 2 * sms)] * 4 + [(1, 3 * sms)]
