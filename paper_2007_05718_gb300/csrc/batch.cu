@@ -36,22 +36,30 @@ struct Group {
   int Ni = 0, dpt = 0, zc = 0;
   // resident CTAs per SM of the batched kernels: [alternative kernel][flux terms]
   int per_sm[2][2] = {{0, 0}, {0, 0}};
-  int zchunk = 16;        // planes per tile
-  // autotuner: candidates are timed on successive ticks of a new member set
+  // autotuner: candidates are timed on successive ticks of a new member set,
+  // once without and once with flux terms (some member has lambda != 0), which
+  // are different kernels: [flux terms]
+  struct Tune {
+    int zchunk = 16;           // planes per tile
+    std::vector<double> cost;  // ms per (site x step) of each candidate
+    int cand = 0;
+    bool tuned = false;
+    long long tuned_sites = 0;
+    int alt = 0;     // 1: the alternative kernel is in use (never with the flux terms)
+    int stage = 0;   // tuning: 0 z chunks, 1 the alternative kernel
+  } tune[2];
+  int flux = 0;  // of the last tick with steps of the group
+  Tune& now() { return tune[flux]; }
+  const Tune& now() const { return tune[flux]; }
   std::vector<int> cands;
-  std::vector<double> cost;  // ms per (site x step) of each candidate
-  int cand = 0;
-  bool tuned = false;
-  long long tuned_sites = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int ctas = 0;           // CTAs of the last launch
   bool paired = false;    // the last tick ran the group in a launch shared with another group
   // alternative batched kernel of the same layout (batch_alt_zc): its planes
-  // per batch (0: none); alt = 1 while it is in use.  The
-  // autotuner times it at the best z chunk after the z-chunk candidates.
-  int alt_zc = 0, alt = 0;
-  int stage = 0;          // tuning: 0 z chunks, 1 the alternative kernel
-  int zc_now() const { return alt ? alt_zc : zc; }
+  // per batch (0: none).  The autotuner times it at the best z chunk after the
+  // z-chunk candidates.  The flux terms have one kernel for both.
+  int alt_zc = 0;
+  int zc_now() const { return now().alt ? alt_zc : zc; }
   int last_zc = 0;        // planes per batch of the kernel of the last launch
 };
 
@@ -98,9 +106,11 @@ struct lb_rt_batch {
   // (mode 2): -1 undecided, 0 separate launches, 1 paired launch, timed on
   // one tick each and normalised per site-direction update
   int pair_a = -1, pair_b = -1, pair_per_sm[2] = {0, 0};  // [flux terms]
-  int pair_choice = -1, pair_trial = 0;
-  long long pair_sites = 0;  // sites of the two groups when the choice was timed
-  double pair_cost[2] = {0.0, 0.0};
+  struct PairTune {
+    int choice = -1, trial = 0;
+    long long sites = 0;  // of the two groups when the choice was timed
+    double cost[2] = {0.0, 0.0};
+  } pair_tune[2];  // [flux terms]
   cudaEvent_t pev0 = nullptr, pev1 = nullptr;
   std::string msg;
 };
@@ -314,13 +324,13 @@ lb_rt_status lb_rt_batch_admit(lb_rt_batch* b, const lb_rt_config* cfg, const lb
       return bcuda(b, e, "batched kernel occupancy");
     }
     for (int z : kZCandidates) g.cands.push_back(z);
-    g.cost.assign(g.cands.size() + 1, 0.0);  // z chunks, then the alternative kernel
+    for (Group::Tune& t : g.tune) t.cost.assign(g.cands.size() + 1, 0.0);  // z chunks, then the alternative kernel
     g.alt_zc = batch_alt_zc(g.dpt, g.zc);
     if (g.alt_zc && query(1) != cudaSuccess) {
       (void)cudaGetLastError();
       g.alt_zc = 0;
     }
-    if (!b->cfg.autotune) g.tuned = true;
+    for (Group::Tune& t : g.tune) t.tuned = !b->cfg.autotune;
     b->groups.push_back(g);
     gi = (int)b->groups.size() - 1;
   }
@@ -347,10 +357,12 @@ lb_rt_status lb_rt_batch_admit(lb_rt_batch* b, const lb_rt_config* cfg, const lb
   Group& grp = b->groups[gi];
   if (grp.alt_zc && h->grid.nz < grp.alt_zc) {
     grp.alt_zc = 0;
-    grp.alt = 0;
-    if (grp.stage == 1) {
-      grp.stage = 0;
-      grp.tuned = true;
+    for (Group::Tune& t : grp.tune) {
+      t.alt = 0;
+      if (t.stage == 1) {
+        t.stage = 0;
+        t.tuned = true;
+      }
     }
   }
   // tensor maps of both parities (for the alternative kernel too, whose
@@ -418,19 +430,20 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     if (!group_sd[g]) continue;
     long long sites = 0;
     for (int s : plan[0][g]) sites += b->slots[s].h->grid.sites;
-    if (b->cfg.autotune && gr.tuned &&
-        (sites > 2 * gr.tuned_sites || 2 * sites < gr.tuned_sites)) {
-      gr.tuned = false;
-      gr.cand = 0;
-      gr.stage = 0;
+    gr.flux = group_flux[g];
+    Group::Tune& t = gr.now();
+    if (b->cfg.autotune && t.tuned && (sites > 2 * t.tuned_sites || 2 * sites < t.tuned_sites)) {
+      t.tuned = false;
+      t.cand = 0;
+      t.stage = 0;
     }
-    if (!gr.tuned) {
-      if (gr.stage == 0) {
-        gr.zchunk = gr.cands[gr.cand];
-        gr.alt = 0;
-        if (gr.cand == 0) gr.tuned_sites = sites;
+    if (!t.tuned) {
+      if (t.stage == 0) {
+        t.zchunk = gr.cands[t.cand];
+        t.alt = 0;
+        if (t.cand == 0) t.tuned_sites = sites;
       } else {
-        gr.alt = 1;  // the alternative kernel at the best z chunk
+        t.alt = 1;  // the alternative kernel at the best z chunk
       }
       tuning = true;
     }
@@ -468,10 +481,11 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     b->pair_b = pb;
     b->pair_per_sm[0] = per_sm[0];
     b->pair_per_sm[1] = per_sm[1];
-    b->pair_choice = -1;
-    b->pair_trial = 0;
+    b->pair_tune[0] = b->pair_tune[1] = lb_rt_batch::PairTune{};
   }
-  const int pair_per_sm = pa >= 0 ? b->pair_per_sm[group_flux[pa] || group_flux[pb]] : 0;
+  const int pair_flux = pa >= 0 && (group_flux[pa] || group_flux[pb]);
+  const int pair_per_sm = pa >= 0 ? b->pair_per_sm[pair_flux] : 0;
+  lb_rt_batch::PairTune& pt = b->pair_tune[pair_flux];
   if (pair_per_sm < 1) pa = pb = -1;
   bool pair_timed = false;  // this tick is one of mode 2's two trials
   if (pa >= 0 && b->cfg.pair_groups == 2) {
@@ -479,22 +493,22 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     long long sites = 0;
     for (int g : {pa, pb})
       for (int s : plan[0][g]) sites += b->slots[s].h->grid.sites;
-    if (b->pair_choice >= 0 && (sites > 2 * b->pair_sites || 2 * sites < b->pair_sites)) {
-      b->pair_choice = -1;
-      b->pair_trial = 0;
+    if (pt.choice >= 0 && (sites > 2 * pt.sites || 2 * sites < pt.sites)) {
+      pt.choice = -1;
+      pt.trial = 0;
     }
-    if (b->pair_choice < 0 && b->pair_trial == 0) b->pair_sites = sites;
-    if (b->pair_choice < 0) {
+    if (pt.choice < 0 && pt.trial == 0) pt.sites = sites;
+    if (pt.choice < 0) {
       pair_timed = true;
-      if (b->pair_trial == 0) pa = pb = -1;  // first trial: separate launches
-    } else if (b->pair_choice == 0) {
+      if (pt.trial == 0) pa = pb = -1;  // first trial: separate launches
+    } else if (pt.choice == 0) {
       pa = pb = -1;
     }
   }
-  if (pa >= 0 && (group_flux[pa] || group_flux[pb])) group_flux[pa] = group_flux[pb] = 1;  // one kernel
+  if (pa >= 0 && pair_flux) group_flux[pa] = group_flux[pb] = 1;  // one kernel
   for (int g = 0; g < G; ++g) {
     const Group& gr = b->groups[g];
-    group_maps[g] = gr.alt;
+    group_maps[g] = gr.now().alt;
     if (group_flux[g] && gr.zc != static_flux_zc(gr.dpt)) {
       if (gr.alt_zc != static_flux_zc(gr.dpt))
         return bfail(b, LB_RT_ECUDA, "no tensor maps for the flux terms of this tile plan");
@@ -549,7 +563,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
         d.collision = h->cfg.collision;
         d.lambda_iters = h->cfg.lambda_iters;
         const int march = march_length(h->grid);
-        d.nzc = std::max(1, std::min(march, (march + gr.zchunk - 1) / gr.zchunk));
+        d.nzc = std::max(1, std::min(march, (march + gr.now().zchunk - 1) / gr.now().zchunk));
         d.tile_start = L.ntiles;
         d.ntiles = static_tiles(h->grid, d.nzc);
         d.budget_partials = nullptr;
@@ -592,7 +606,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     }
     for (size_t i = first_of_step; i < launches.size(); ++i) {
       const Launch& L = launches[i];
-      for (long long v : {(long long)L.group, (long long)group_maps[L.group], (long long)b->groups[L.group].alt,
+      for (long long v : {(long long)L.group, (long long)group_maps[L.group], (long long)b->groups[L.group].now().alt,
                           (long long)L.first, (long long)L.nprob,
                           (long long)L.ntiles, (long long)L.flux, (long long)L.b_group,
                           (long long)L.b_first, (long long)L.b_nprob, (long long)L.b_ntiles,
@@ -627,7 +641,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       B.N = gr.Ni;
       B.dpt = gr.dpt;
       B.zc = gr.zc_now();
-      B.alt = gr.alt;
+      B.alt = gr.now().alt;
       B.storage = b->cfg.storage;
       B.ctas = ctas;
       B.flux = flux;
@@ -635,11 +649,12 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
       B.sched = b->d_err + 1;
       return B;
     };
+    auto planes = [&](const Group& gr, int flux) { return flux ? static_flux_zc(gr.dpt) : gr.zc_now(); };
     auto single = [&](const Launch& L) -> cudaError_t {
       Group& gr = b->groups[L.group];
-      const int per_sm = gr.per_sm[gr.alt][L.flux];
+      const int per_sm = gr.per_sm[gr.now().alt][L.flux];
       const int ctas = (int)std::min<long long>((long long)per_sm * b->sms, L.ntiles);
-      gr.last_zc = gr.zc_now();
+      gr.last_zc = planes(gr, L.flux);
       gr.ctas = ctas;
       gr.paired = false;
       return launch_static_batch(batch_of(L.group, L.first, L.nprob, L.ntiles, L.flux, ctas),
@@ -648,7 +663,7 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     if (timed && tuning) {
       for (int g = 0; g < G && e == cudaSuccess; ++g) {
         Group& gr = b->groups[g];
-        const bool time_it = !gr.tuned && group_sd[g] > 0;
+        const bool time_it = !gr.now().tuned && group_sd[g] > 0;
         if (time_it) e = cudaEventRecord(gr.ev0, b->stream);
         for (const Launch& L : launches)
           if (L.group == g && e == cudaSuccess) e = single(L);
@@ -670,8 +685,8 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
           batch_of(L.b_group, L.b_first, L.b_nprob, L.b_ntiles, L.b_flux, L.ctas - L.ctas_a);
       ga.ctas = L.ctas_a;
       gb.ctas = L.ctas - L.ctas_a;
-      ga.last_zc = ga.zc_now();
-      gb.last_zc = gb.zc_now();
+      ga.last_zc = planes(ga, L.flux);
+      gb.last_zc = planes(gb, L.b_flux);
       ga.paired = gb.paired = true;
       e = launch_static_batch_pair(A, ga.table, B, gb.table, L.ctas_a, L.ctas, b->stream);
     }
@@ -733,37 +748,38 @@ lb_rt_status lb_rt_batch_tick(lb_rt_batch* b, int* n_active) {
     BCK(b, cudaEventElapsedTime(&ms, b->pev0, b->pev1));
     long long sd = 0;
     for (int g = 0; g < G; ++g) sd += group_sd[g] * b->groups[g].Ni;
-    b->pair_cost[b->pair_trial] = sd ? ms / (double)sd : 0.0;
-    if (++b->pair_trial == 2) b->pair_choice = b->pair_cost[1] < b->pair_cost[0] ? 1 : 0;
+    pt.cost[pt.trial] = sd ? ms / (double)sd : 0.0;
+    if (++pt.trial == 2) pt.choice = pt.cost[1] < pt.cost[0] ? 1 : 0;
   }
   if (tuning) {
     BCK(b, cudaStreamSynchronize(b->stream));
     for (int g = 0; g < G; ++g) {
       Group& gr = b->groups[g];
-      if (gr.tuned || !group_sd[g]) continue;
+      if (!group_sd[g] || gr.now().tuned) continue;
+      Group::Tune& t = gr.now();
       float ms = 0.f;
       BCK(b, cudaEventElapsedTime(&ms, gr.ev0, gr.ev1));
       const int nz = (int)gr.cands.size();
-      if (gr.stage == 1) {
+      if (t.stage == 1) {
         // keep the alternative kernel only if it beat the best z chunk
-        gr.cost[nz] = ms / (double)group_sd[g];
-        double best = gr.cost[0];
-        for (int i = 1; i < nz; ++i) best = std::min(best, gr.cost[i]);
-        gr.alt = gr.cost[nz] < best ? 1 : 0;
-        gr.stage = 0;
-        gr.tuned = true;
+        t.cost[nz] = ms / (double)group_sd[g];
+        double best = t.cost[0];
+        for (int i = 1; i < nz; ++i) best = std::min(best, t.cost[i]);
+        t.alt = t.cost[nz] < best ? 1 : 0;
+        t.stage = 0;
+        t.tuned = true;
         continue;
       }
-      gr.cost[gr.cand] = ms / (double)group_sd[g];
-      if (++gr.cand == nz) {
+      t.cost[t.cand] = ms / (double)group_sd[g];
+      if (++t.cand == nz) {
         int best = 0;
         for (int i = 1; i < nz; ++i)
-          if (gr.cost[i] < gr.cost[best]) best = i;
-        gr.zchunk = gr.cands[best];
-        if (gr.alt_zc) {
-          gr.stage = 1;
+          if (t.cost[i] < t.cost[best]) best = i;
+        t.zchunk = gr.cands[best];
+        if (gr.alt_zc && !gr.flux) {
+          t.stage = 1;
         } else {
-          gr.tuned = true;
+          t.tuned = true;
         }
       }
     }
@@ -844,7 +860,7 @@ lb_rt_status lb_rt_batch_plan(const lb_rt_batch* b, int slot, int* dirs_per_warp
 lb_rt_status lb_rt_batch_tuning(const lb_rt_batch* b, int slot, int* zchunk, int* ctas) {
   if (!b || slot < 0 || slot >= (int)b->slots.size() || !b->slots[slot].used) return LB_RT_EINVAL;
   const Group& g = b->groups[b->slots[slot].group];
-  if (zchunk) *zchunk = g.zchunk;
+  if (zchunk) *zchunk = g.now().zchunk;
   if (ctas) *ctas = g.ctas;
   return LB_RT_OK;
 }

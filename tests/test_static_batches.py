@@ -124,3 +124,40 @@ def test_every_batched_kernel_gets_its_own_residency(cuda):
     finally:
         lbrt.lb_rt_batch_destroy(b)
     assert seen == [(2, 2 * sms)] * 4 + [(1, 3 * sms)]
+
+
+def test_tuning_and_plan_follow_the_flux_terms(cuda):
+    """The flux terms (lambda != 0 somewhere in the group) take one plane a batch
+    and have no alternative kernel to time; a tile shape chosen with them is not
+    kept once they are gone."""
+    b = lbrt.lb_rt_batch_create(max_problems=2, storage=F32, steps_per_tick=1)
+    try:
+        prob = dict(dims=3, nx=64, ny=16, nz=64, **ICO[1])
+        E0 = W.random_fields((64, 16, 64), 1)
+        lbrt.lb_rt_batch_admit(b, prob, dict(kappa_0=2.0, lam=0.3), E0, lbrt.LB_RT_STATE_ISOTROPIC, 6)
+        s = lbrt.lb_rt_batch_admit(b, prob, dict(kappa_0=2.0), E0, lbrt.LB_RT_STATE_ISOTROPIC, 100)
+        planes = []
+        for _ in range(11):
+            lbrt.lb_rt_batch_tick(b)
+            planes.append(lbrt.lb_rt_batch_plan(b, s)[1])
+        lbrt.lb_rt_batch_sync(b)
+    finally:
+        lbrt.lb_rt_batch_destroy(b)
+    # six ticks with the flux terms; then four z chunks and the alternative kernel
+    assert planes == [1] * 6 + [2] * 4 + [1]
+
+
+def test_flux_terms_do_not_keep_groups_from_pairing(cuda):
+    b = lbrt.lb_rt_batch_create(max_problems=2, storage=F32, steps_per_tick=1, pair_groups=1)
+    try:
+        E0 = W.random_fields((16, 16, 64), 1)
+        s = [lbrt.lb_rt_batch_admit(b, dict(dims=3, nx=64, ny=16, nz=16, **ICO[l]), dict(kappa_0=2.0, lam=0.3),
+                                    E0, lbrt.LB_RT_STATE_ISOTROPIC, 100) for l in (1, 2)]
+        paired = []
+        for _ in range(6):
+            lbrt.lb_rt_batch_tick(b)
+            paired.append([lbrt.lb_rt_batch_plan(b, k)[2] for k in s])
+        lbrt.lb_rt_batch_sync(b)
+    finally:
+        lbrt.lb_rt_batch_destroy(b)
+    assert paired == [[0, 0]] * 4 + [[1, 1]] * 2
