@@ -161,3 +161,21 @@ def test_flux_terms_do_not_keep_groups_from_pairing(cuda):
     finally:
         lbrt.lb_rt_batch_destroy(b)
     assert paired == [[0, 0]] * 4 + [[1, 1]] * 2
+
+
+@pytest.mark.parametrize("storage", [F32, F16, BF16])
+@pytest.mark.parametrize("lams", [(0.3, 0.0), (0.0, 0.3), (0.3, 0.3)], ids=str)
+def test_paired_launch_with_flux_terms(cuda, storage, lams):
+    """A lambda in either group puts both on the flux terms of the paired kernel,
+    the 42-direction group on its one-plane boxes."""
+    probs = []
+    for k, (shape, level, ndir) in enumerate([((9, 5, 63), 1, 42), ((12, 3, 65), 2, 162), ((17, 4, 64), 1, 42),
+                                              ((3, 7, 130), 2, 162)]):
+        probs.append(dict(dims=3, shape=shape, dirs=ICO[level], bc=(P, V, P), state=W.random_populations(ndir, shape, k),
+                          fluid=dict(kappa_a=0.5, kappa_0=3.0, eta=W.random_fields(shape, 9 + k),
+                                     lam=lams[0] if level == 1 and k == 0 else lams[1] if level == 2 and k == 1 else 0.0)))
+    got, plans = _batch(probs, storage, 5, pair_groups=1)
+    assert plans == [(5, 1, 1), (11, 1, 1)] * 2
+    for p, (E, F) in zip(probs, got):
+        E1, F1 = _alone(p, storage, 5)
+        assert np.isfinite(E1).all() and np.array_equal(E, E1) and np.array_equal(F, F1)
