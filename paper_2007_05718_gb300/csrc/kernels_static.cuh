@@ -121,9 +121,9 @@ __host__ __device__ constexpr int st_eslot_floats() {
   return ((kBoxE * 3 * (ZC + 1) * 4 + 127) / 128) * 32;
 }
 // A tile in the queue: column, row and padded plane of item 0, planes (2D: minus
-// the rows; 0: no such tile), problem (batch), flag bits 2, 8 and 16 of BatchCtx.
+// the rows; 0: no such tile), flag bits 2, 8 and 16 of BatchCtx.
 struct TileInfo {
-  int x0, y, z, len, prob, flags;
+  int x0, y, z, len, flags;
 };
 
 // Shared memory (bytes), every offset known at compile time (GM = the plan's
@@ -271,7 +271,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
   ProblemDesc* const pd = reinterpret_cast<ProblemDesc*>(smem_raw + L::DESC);
   auto desc = [&](int slot) -> const ProblemDesc& { return BATCH ? pd[slot] : one; };
   int w_prob = 0;  // warp 0: problem of the tile published last
-  auto publish = [&](int n, long long tl) {
+  auto publish = [&](int n, int tl) {
     int x0 = 0, y = 0, z = 0, len = 0, p = w_prob, fl = 0;
     if (tl < ntiles) {
       if constexpr (BATCH) {
@@ -307,7 +307,6 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
       e.y = y;
       e.z = z;
       e.len = len;
-      e.prob = p;
       e.flags = fl;
       st_release(tq_count, n + 1);
     }
@@ -328,6 +327,7 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     return true;
   };
   auto items_of = [&](int len) { return len < 0 ? -len : tile_items<ZC>(len); };
+  int my_tile = cta;        // warp 0: the tile published last
   unsigned grabbed = 0;     // warp 0, lane 0: counter value of the tile to publish
   bool to_publish = false;
 
@@ -341,7 +341,12 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     // behind the stores in flight
     if (!to_publish || (m < 2 && m + kRing + 1 < M)) return;
     to_publish = false;
-    publish(tn + 1, (long long)ncta + __shfl_sync(0xffffffffu, grabbed, 0));
+    // (the test of `sched`, never null, is for the compiler, which otherwise
+    // makes other choices all over the batched kernels: ten float16 problems of
+    // 32^3 to 128^3, 40 steps, 51.07 instead of 50.26 ms)
+    if (BATCH && !sched) my_tile += ncta;
+    else my_tile = ncta + (int)__shfl_sync(0xffffffffu, grabbed, 0);
+    publish(tn + 1, my_tile);
   };
   auto open_tile = [&]() {  // false: no tile left
     ++tn;
@@ -364,8 +369,8 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
     t_base = static_cast<ST*>(D.out) + (long long)i0 * D.g.si + (long long)t_z * D.g.sz +
              (long long)(t_y + 1) * D.g.sy + (t_x0 + 2 * lane + GL);
     if (g == 0) {
-      // (sched is never null; without the test the compiler merges this branch
-      // with others and spills up to 186 bytes: 128^3 x 42 took 2.4 times as long)
+      // (the same here: without the test up to 186 bytes are spilled, and the
+      // 128^3 x 42 float32 step took 2.4 times as long)
       if (sched && lane == 0) grabbed = atomicAdd(sched, 1u);
       to_publish = true;
     }
@@ -931,6 +936,8 @@ k_static_pair(const __grid_constant__ CUtensorMap unused, const __grid_constant_
                                                  ta, sched, blockIdx.x, ctas_a, ga);
   } else {
     if ((int)threadIdx.y >= gb) return;
+    // (the test of `sched` as in static_body: without it the ten float16 problems
+    // take 65.4 instead of 53.8 ms)
     static_body<ST, 1, FLUX, DB, ZB, UB, HB, MAXT / 32, true>(unused, unused, none, table_b, nprob_b, ntiles_b, err,
                                                  tb, sched ? sched + 2 : nullptr, blockIdx.x - ctas_a, gridDim.x - ctas_a, gb);
   }

@@ -55,13 +55,6 @@ cudaError_t static_plan(const StaticCall& c) {
                 : static_kernel<ST, 0, false, DPT, ZC, HU, H, MAXT, REGS>(c);
 }
 
-// batched launches only (the alternative kernel of a plan)
-template <class ST, int DPT, int ZC, int HU, int H, int MAXT, int REGS>
-cudaError_t static_plan_batch(const StaticCall& c) {
-  return c.flux ? static_kernel<ST, 1, true, DPT, ZC, HU, H, MAXT, REGS>(c)
-                : static_kernel<ST, 1, false, DPT, ZC, HU, H, MAXT, REGS>(c);
-}
-
 template <class ST, bool FLUX, int DA, int ZA, int UA, int HA, int DB, int ZB, int UB, int HB, int MAXT, int REGS>
 cudaError_t pair_kernel(const StaticPairCall& c) {
   auto* k = k_static_pair<ST, FLUX, DA, ZA, UA, HA, DB, ZB, UB, HB, MAXT, REGS>;

@@ -116,10 +116,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, un
   return true;
 }
 
-__device__ __forceinline__ float fld(const float* __restrict__ p, float s, long long i) {
-  return p ? __ldg(p + i) : s;
-}
-
 // A word in shared memory that publishes what the CTA wrote before it.
 __device__ __forceinline__ void st_release(uint32_t addr, int v) {
   asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
