@@ -290,14 +290,15 @@ __device__ __forceinline__ bool site_pair(const Grid& g, long long p, SitePair& 
   return true;
 }
 
-// populations (x, x + 1) of a direction row as float32 pair; 16-bit storage:
-// I = w E^ (1 + q)
+// Populations (x, x + 1) of a direction row, as stored and as a float32 pair;
+// 16-bit storage: I = w E^ (1 + q).
 template <class ST>
-__device__ __forceinline__ float2 load_pair(const ST* p, float2 Eh, float w) {
+using RawPair = std::conditional_t<std::is_same<ST, float>::value, float2, unsigned>;
+template <class ST>
+__device__ __forceinline__ float2 decode_pair(RawPair<ST> v, float2 Eh, float w) {
   if constexpr (std::is_same<ST, float>::value) {
-    return *reinterpret_cast<const float2*>(p);
+    return v;
   } else {
-    const unsigned v = *reinterpret_cast<const unsigned*>(p);
     ST lo, hi;
     const unsigned short a = (unsigned short)v, b = (unsigned short)(v >> 16);
     memcpy(&lo, &a, 2);
@@ -308,7 +309,8 @@ __device__ __forceinline__ float2 load_pair(const ST* p, float2 Eh, float w) {
 
 // Moments of a site pair: sums over directions in the table order.  The rows
 // of padding and, past the end of an odd row, the ghost column are read and
-// not used.
+// not used.  U > 1: U directions are loaded before any is added up (left to
+// itself the compiler keeps too few loads in flight where there are ten sums).
 struct Moments {
   float e = 0, fx = 0, fy = 0, fz = 0, pxx = 0, pxy = 0, pxz = 0, pyy = 0, pyz = 0, pzz = 0;
   template <bool WITH_P>
@@ -328,7 +330,7 @@ struct Moments {
   }
 };
 
-template <class ST, bool WITH_P>
+template <class ST, bool WITH_P, int U>
 __device__ __forceinline__ void pair_moments(const Grid& g, int N, const ST* __restrict__ pop,
                                              const float* __restrict__ e, const DirTable& t, const SitePair& q,
                                              Moments& a, Moments& b) {
@@ -336,19 +338,33 @@ __device__ __forceinline__ void pair_moments(const Grid& g, int N, const ST* __r
   if constexpr (!std::is_same<ST, float>::value)
     Eh = *reinterpret_cast<const float2*>(e + eidx(g, q.z, q.y, q.x));
   const ST* p = pop + pidx(g, 0, q.z, q.y, q.x);
-#pragma unroll 4
-  for (int i = 0; i < N; ++i, p += g.si) {
+  auto add = [&](RawPair<ST> v, int i) {
     const float4 nw = t.nw[i];
-    const float2 v = load_pair<ST>(p, Eh, nw.w);
-    a.add<WITH_P>(nw, v.x);
-    b.add<WITH_P>(nw, v.y);
+    const float2 f = decode_pair<ST>(v, Eh, nw.w);
+    a.add<WITH_P>(nw, f.x);
+    b.add<WITH_P>(nw, f.y);
+  };
+  int i = 0;
+  if constexpr (U > 1) {
+#pragma unroll 1
+    for (; i + U <= N; i += U) {
+      RawPair<ST> v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u, p += g.si) v[u] = *reinterpret_cast<const RawPair<ST>*>(p);
+#pragma unroll
+      for (int u = 0; u < U; ++u) add(v[u], i + u);
+    }
   }
+#pragma unroll 4
+  for (; i < N; ++i, p += g.si) add(*reinterpret_cast<const RawPair<ST>*>(p), i);
 }
 
 // E, F, P of the current populations, two sites a thread: 8-byte (4-byte) loads
 // bring whole sectors, and E and F alone (no P) leave out six of ten sums.
 // 128^3 x 162 float16: 0.42 -> 0.14 ms (5.3 TB/s); 256^3 x 162 float32: 2.4 ->
-// 1.78 ms (6.7 TB/s), the rate of a plain copy.
+// 1.78 ms (6.7 TB/s), the rate of a plain copy.  With P, eight directions loaded
+// ahead: 128^3 x 162 float16 0.43 -> 0.24 ms, 64^3 67 -> 46 us (four, as the
+// compiler places them: 0.41 ms and 87 us).
 template <class ST, bool WITH_P>
 __global__ void k_moments(Grid g, int N, const ST* __restrict__ pop, const float* __restrict__ e,
                           float* __restrict__ E, float* __restrict__ F, float* __restrict__ P,
@@ -356,7 +372,7 @@ __global__ void k_moments(Grid g, int N, const ST* __restrict__ pop, const float
   SitePair q;
   if (!site_pair(g, blockIdx.x * (long long)blockDim.x + threadIdx.x, q)) return;
   Moments m[2];
-  pair_moments<ST, WITH_P>(g, N, pop, e, t, q, m[0], m[1]);
+  pair_moments<ST, WITH_P, WITH_P ? 8 : 1>(g, N, pop, e, t, q, m[0], m[1]);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     if (k && !q.in1) return;
@@ -458,7 +474,9 @@ __global__ void k_total_partials16(Grid g, int N, const ST* __restrict__ pop,
 // H^0 = v.H the time component of the comoving flux (H^mu u_mu = 0,
 // signature -+++).  ST = float: populations; 16-bit types: the deviation
 // form against the E array `e`.  Two sites a thread, bound by the latency of
-// the loads at small grids: 64^3 x 42 float32, 20.7 -> 15.0 us.
+// the loads at small grids: 64^3 x 42 float32, 16.7 -> 12.7 us.  Eight directions
+// loaded ahead pay from about a hundred directions on: 64^3 x 162 float16 48 ->
+// 42 us, but 128^3 x 42 float32 94 -> 101.
 template <class ST>
 __global__ void k_coupling(Grid g, int N, const ST* __restrict__ pop, const float* __restrict__ e,
                            const __grid_constant__ DirTable t, MovingCoef c, float* __restrict__ Jo,
@@ -466,7 +484,8 @@ __global__ void k_coupling(Grid g, int N, const ST* __restrict__ pop, const floa
   SitePair q;
   if (!site_pair(g, blockIdx.x * (long long)blockDim.x + threadIdx.x, q)) return;
   Moments mm[2];
-  pair_moments<ST, true>(g, N, pop, e, t, q, mm[0], mm[1]);
+  if (N >= 96) pair_moments<ST, true, 8>(g, N, pop, e, t, q, mm[0], mm[1]);
+  else pair_moments<ST, true, 1>(g, N, pop, e, t, q, mm[0], mm[1]);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     if (k && !q.in1) return;
@@ -513,7 +532,12 @@ __global__ void k_coupling(Grid g, int N, const ST* __restrict__ pop, const floa
 }
 
 unsigned grid1d(long long n) { return (unsigned)((n + BLK - 1) / BLK); }
-unsigned pair_grid(const Grid& g) { return grid1d((long long)((g.nx + 1) / 2) * g.ny * g.nz); }
+// blocks of the kernels that take two sites a thread; of 128 threads, so that a
+// small grid still reaches every SM (31^3 x 42: coupling 8.4 -> 7.6 us)
+constexpr int PAIR_BLK = 128;
+unsigned pair_grid(const Grid& g) {
+  return (unsigned)(((long long)((g.nx + 1) / 2) * g.ny * g.nz + PAIR_BLK - 1) / PAIR_BLK);
+}
 
 }  // namespace
 
@@ -537,8 +561,8 @@ cudaError_t launch_moments(const Grid& g, int N, const void* pop, const float* e
   auto go = [&](auto tag) {
     using ST = decltype(tag);
     const ST* p = static_cast<const ST*>(pop);
-    if (P) k_moments<ST, true><<<pair_grid(g), BLK, 0, s>>>(g, N, p, e, E, F, P, t);
-    else k_moments<ST, false><<<pair_grid(g), BLK, 0, s>>>(g, N, p, e, E, F, P, t);
+    if (P) k_moments<ST, true><<<pair_grid(g), PAIR_BLK, 0, s>>>(g, N, p, e, E, F, P, t);
+    else k_moments<ST, false><<<pair_grid(g), PAIR_BLK, 0, s>>>(g, N, p, e, E, F, P, t);
   };
   if (storage == ST_F32) go(float());
   else if (storage == ST_F16) go(__half());
@@ -582,13 +606,13 @@ cudaError_t launch_coupling(const Grid& g, int N, const void* pop, const float* 
                             const DirTable& t, const MovingCoef& c, float* J, float* H, float* S,
                             cudaStream_t s) {
   if (storage == ST_F32)
-    k_coupling<float><<<pair_grid(g), BLK, 0, s>>>(g, N, static_cast<const float*>(pop), e, t,
+    k_coupling<float><<<pair_grid(g), PAIR_BLK, 0, s>>>(g, N, static_cast<const float*>(pop), e, t,
                                                       c, J, H, S);
   else if (storage == ST_F16)
-    k_coupling<__half><<<pair_grid(g), BLK, 0, s>>>(g, N, static_cast<const __half*>(pop), e,
+    k_coupling<__half><<<pair_grid(g), PAIR_BLK, 0, s>>>(g, N, static_cast<const __half*>(pop), e,
                                                        t, c, J, H, S);
   else
-    k_coupling<__nv_bfloat16><<<pair_grid(g), BLK, 0, s>>>(
+    k_coupling<__nv_bfloat16><<<pair_grid(g), PAIR_BLK, 0, s>>>(
         g, N, static_cast<const __nv_bfloat16*>(pop), e, t, c, J, H, S);
   return cudaGetLastError();
 }

@@ -9,9 +9,7 @@ namespace lbrt {
 
 cudaError_t static_bf16_d5(const StaticCall& c) {
   if (c.flux || c.alt || c.zc == 1) return static_plan<__nv_bfloat16, 5, 1, 2, 5, 320, 96>(c);
-  if (c.budget) return static_kernel<__nv_bfloat16, 4, false, 5, 2, 1, 2, 320, 96>(c);
-  return c.mode == 1 ? static_kernel<__nv_bfloat16, 1, false, 5, 2, 1, 2, 320, 96>(c)
-                     : static_kernel<__nv_bfloat16, 0, false, 5, 2, 1, 2, 320, 96>(c);
+  return static_plain<__nv_bfloat16, 5, 2, 1, 2, 320, 96>(c);
 }
 
 cudaError_t static_bf16_pair(const StaticPairCall& c) {

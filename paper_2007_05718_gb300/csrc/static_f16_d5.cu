@@ -9,9 +9,7 @@ namespace lbrt {
 
 cudaError_t static_f16_d5(const StaticCall& c) {
   if (c.flux || c.alt || c.zc == 1) return static_plan<__half, 5, 1, 2, 5, 320, 96>(c);
-  if (c.budget) return static_kernel<__half, 4, false, 5, 2, 1, 2, 320, 96>(c);
-  return c.mode == 1 ? static_kernel<__half, 1, false, 5, 2, 1, 2, 320, 96>(c)
-                     : static_kernel<__half, 0, false, 5, 2, 1, 2, 320, 96>(c);
+  return static_plain<__half, 5, 2, 1, 2, 320, 96>(c);
 }
 
 cudaError_t static_f16_pair(const StaticPairCall& c) {

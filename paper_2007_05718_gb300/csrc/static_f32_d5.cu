@@ -8,11 +8,9 @@
 namespace lbrt {
 
 cudaError_t static_f32_d5(const StaticCall& c) {
-  if (c.alt && !c.flux) return static_kernel<float, 1, false, 5, 1, 1, 2, 320, 72>(c);
-  if (c.mode == 2 || c.flux || c.zc == 1) return static_plan<float, 5, 1, 2, 5, 320, 96>(c);
-  if (c.budget) return static_kernel<float, 4, false, 5, 2, 1, 5, 320, 96>(c);
-  return c.mode == 1 ? static_kernel<float, 1, false, 5, 2, 1, 5, 320, 96>(c)
-                     : static_kernel<float, 0, false, 5, 2, 1, 5, 320, 96>(c);
+  if (c.flux || c.mode == 2) return static_flux<float, 5, 1, 0, 2, 320, 72>(c);
+  if (c.alt) return static_kernel<float, 1, false, 5, 1, 1, 2, 320, 72>(c);
+  return c.zc == 1 ? static_plain<float, 5, 1, 2, 5, 320, 96>(c) : static_plain<float, 5, 2, 1, 5, 320, 96>(c);
 }
 
 cudaError_t static_f32_pair(const StaticPairCall& c) {

@@ -204,6 +204,14 @@ cudaError_t occupancy_static_batch_pair(int storage, int dpt_a, int zc_a, int Na
 // is about the mean of the evenly shared work and of the busiest SM's whole
 // tiles, plus half a tile for the end of the launch.  A tile's work is its
 // batches (a 3D tile of l planes loads l + 1, rounded up to whole batches).
+// Kernels with the flux terms, and those of three or more small CTAs an SM, go
+// by the busiest CTA instead: they are bound by the latency of a batch's chain,
+// which the CTAs of an SM go through side by side, and want shorter tiles (us a
+// step: 64^3 x 12 with the flux terms 37 -> 29, 64^3 x 42 48 -> 46, 93x61x47 x 72
+// 98 -> 91, 100^3 x 12 110 -> 95).  For two CTAs an SM without the flux terms that
+// would be faster alone (64^3 x 42 51 -> 42) but slower beside the steps of other
+// handles, which fill the ends of a launch (three 128^3 x 42 spheres 2.5 %, three
+// 96x49x33 x 42 bfloat16 problems 13 %): the planes read twice are work.
 //
 // Moving step: tiles cta, cta + ncta, ...; the count minimises the busiest
 // CTA's share of plane loads.
@@ -237,6 +245,7 @@ cudaError_t plan_static_grid(const Grid& g, int Ni, int dpt, int zc, int storage
     const long long plane = 64LL * Ni * (storage == ST_F32 ? 4 : 2) * per_sm;
     const int longest = (int)std::max(8LL, (720LL << 10) / plane);
     const int fewest = flat ? 1 : std::min((march + longest - 1) / longest, 512);
+    const long long share = flux || per_sm >= 3 ? slots : sms;
     double best = 1e300;
     *nzc = 1;
     for (int c = fewest; c <= std::min(march, 512) && columns * c <= (1LL << 24); ++c) {
@@ -244,8 +253,8 @@ cudaError_t plan_static_grid(const Grid& g, int Ni, int dpt, int zc, int storage
       auto items = [&](int len) { return flat ? len : (len + 1 + zc - 1) / zc; };
       const double most = items(base + (rem ? 1 : 0));
       const double total = (double)columns * ((double)rem * items(base + 1) + (double)(c - rem) * items(base));
-      const double whole = (double)((columns * c + sms - 1) / sms) * (total / ((double)columns * c));
-      const double cost = 0.5 * (total / sms + whole) + 0.5 * most;
+      const double whole = (double)((columns * c + share - 1) / share) * (total / ((double)columns * c));
+      const double cost = 0.5 * (total / share + whole) + 0.5 * most;
       if (cost < best * 0.999) {
         best = cost;
         *nzc = c;

@@ -38,21 +38,31 @@ cudaError_t static_kernel(const StaticCall& c) {
   return cudaGetLastError();
 }
 
+// kernels of a plan with the flux terms
 template <class ST, int DPT, int ZC, int HU, int H, int MAXT, int REGS>
-cudaError_t static_plan(const StaticCall& c) {
-  if (c.mode == 1)
-    return c.flux ? static_kernel<ST, 1, true, DPT, ZC, HU, H, MAXT, REGS>(c)
-                  : static_kernel<ST, 1, false, DPT, ZC, HU, H, MAXT, REGS>(c);
+cudaError_t static_flux(const StaticCall& c) {
+  if (c.mode == 1) return static_kernel<ST, 1, true, DPT, ZC, HU, H, MAXT, REGS>(c);
   if constexpr (SV<ST>::F32) {
     if (c.mode == 2)
       return c.budget ? static_kernel<ST, 2 + 4, true, DPT, ZC, HU, H, MAXT, REGS>(c)
                       : static_kernel<ST, 2, true, DPT, ZC, HU, H, MAXT, REGS>(c);
   }
-  if (c.budget)
-    return c.flux ? static_kernel<ST, 4, true, DPT, ZC, HU, H, MAXT, REGS>(c)
-                  : static_kernel<ST, 4, false, DPT, ZC, HU, H, MAXT, REGS>(c);
-  return c.flux ? static_kernel<ST, 0, true, DPT, ZC, HU, H, MAXT, REGS>(c)
-                : static_kernel<ST, 0, false, DPT, ZC, HU, H, MAXT, REGS>(c);
+  return c.budget ? static_kernel<ST, 4, true, DPT, ZC, HU, H, MAXT, REGS>(c)
+                  : static_kernel<ST, 0, true, DPT, ZC, HU, H, MAXT, REGS>(c);
+}
+
+// and without them
+template <class ST, int DPT, int ZC, int HU, int H, int MAXT, int REGS>
+cudaError_t static_plain(const StaticCall& c) {
+  if (c.mode == 1) return static_kernel<ST, 1, false, DPT, ZC, HU, H, MAXT, REGS>(c);
+  return c.budget ? static_kernel<ST, 4, false, DPT, ZC, HU, H, MAXT, REGS>(c)
+                  : static_kernel<ST, 0, false, DPT, ZC, HU, H, MAXT, REGS>(c);
+}
+
+template <class ST, int DPT, int ZC, int HU, int H, int MAXT, int REGS>
+cudaError_t static_plan(const StaticCall& c) {
+  return c.flux || c.mode == 2 ? static_flux<ST, DPT, ZC, HU, H, MAXT, REGS>(c)
+                               : static_plain<ST, DPT, ZC, HU, H, MAXT, REGS>(c);
 }
 
 template <class ST, bool FLUX, int DA, int ZA, int UA, int HA, int DB, int ZB, int UB, int HB, int MAXT, int REGS>
