@@ -61,15 +61,18 @@ def _peaks():
 
 CSRC = os.path.join(ROOT, "paper_2007_05718_gb300", "csrc")
 # the ncu summary of each timed kernel (traffic per launch, scaled to the
-# bench size where the summary says so) and the sources it was captured from
+# bench size where the summary says so) and the sources that decide what was
+# captured: the kernel, its instance (planes, look-ahead, registers) and the
+# tile plan with the grid
+_STATIC = ("kernels_static.cuh", "tma_common.cuh", "static_unit.cuh", "static_step.cu")
 PROFILES = {
-    "c3_fp32": ("step_static_f32_diffusion256_162.md", ("kernels_static.cuh", "tma_common.cuh")),
-    "c3_fp16": ("step_static_f16_diffusion256_162.md", ("kernels_static.cuh", "tma_common.cuh")),
-    "c3_bf16": ("step_static_bf16_diffusion256_162.md", ("kernels_static.cuh", "tma_common.cuh")),
-    "c2_fp32": ("step_static_f32_sphere128_42.md", ("kernels_static.cuh", "tma_common.cuh")),
-    "c2_fp16": ("step_static_f16_sphere128_42.md", ("kernels_static.cuh", "tma_common.cuh")),
-    "c5_fp32": ("step_moving_f32_shear128_162.md", ("kernels_tma_moving.cu", "tma_common.cuh")),
-    "c5_fp16": ("step_moving_f16_shear128_162.md", ("kernels_moving16.cu", "tma_common.cuh")),
+    "c3_fp32": ("step_static_f32_diffusion256_162.md", _STATIC + ("static_f32_d11.cu",)),
+    "c3_fp16": ("step_static_f16_diffusion256_162.md", _STATIC + ("static_f16_d11.cu",)),
+    "c3_bf16": ("step_static_bf16_diffusion256_162.md", _STATIC + ("static_bf16_d11.cu",)),
+    "c2_fp32": ("step_static_f32_sphere128_42.md", _STATIC + ("static_f32_d5.cu",)),
+    "c2_fp16": ("step_static_f16_sphere128_42.md", _STATIC + ("static_f16_d5.cu",)),
+    "c5_fp32": ("step_moving_f32_shear128_162.md", ("kernels_tma_moving.cu", "tma_common.cuh", "static_step.cu")),
+    "c5_fp16": ("step_moving_f16_shear128_162.md", ("kernels_moving16.cu", "tma_common.cuh", "static_step.cu")),
 }
 
 
