@@ -48,16 +48,20 @@
 // direction and 64-site plane, issue slots 49 % busy.  Behind DRAM the
 // shared-memory wavefronts of the stream (48 of 59 cycles per direction-plane
 // with resident boxes) are the next limit.  16 bits: the decode and the lerps,
-// 84 instructions, issue slots 70 % busy, 1.16 ms.  Before (partials and
-// scalars between two CTA barriers per plane, tiles dealt out in advance) the
-// same grid took 2.0 and 2.2 ms; step times in ms:
-//   256^3 x 162 float32 7.8 -> 5.0, 16 bits 9.0 -> 4.3
-//   128^3 x 42 float32 0.21 -> 0.16, float16 0.26 -> 0.18
-//   512^2 x 162 float32 sweep 73 -> 12.6 (27 before the mirror planes went)
+// 84 instructions, issue slots 70 % busy, 1.16 ms.  Waiting takes no issue slots
+// worth naming: a launch repeats about 12000 tries of its barriers and queue, in
+// 0.7 to 1.0e9 warp instructions (the hardware suspends a waiting warp).  Before
+// (partials and scalars between two CTA barriers per plane, tiles dealt out in
+// advance) the same grid took 2.0 and 2.2 ms.  Times in ms:
+//   a step, 256^3 x 162, float32 7.5 -> 4.74, float16 8.8 -> 4.30
+//   a step, 128^3 x 42 sphere, float32 0.21 -> 0.15, float16 0.24 -> 0.18
+//   a step of eight 512^2 x 120 float32 problems in a batch 3.63 -> 0.62 (1.32
+//   before the mirror planes went)
 //
-// Every wait is bounded (about 2 s): one that gives up sets the error word,
-// and the warp goes on with stale (in-bounds) data, still arriving at every
-// barrier, so that no other warp is left waiting.
+// Every wait is bounded (about 2 s).  A warp whose wait gives up sets the error
+// word and leaves its loop, after the copies it has in flight have landed; what
+// is left of its tiles is not written.  It no longer arrives at P and C, so the
+// other warps of the CTA run into their own limit and leave likewise.
 #pragma once
 
 #include <algorithm>

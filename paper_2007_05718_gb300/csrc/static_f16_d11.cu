@@ -1,7 +1,7 @@
 // 16-bit storage, 11 directions per warp (the 162-direction icosahedral set).
 // All directions are streamed ahead of the collision scalars: 256^3 x 162,
-// eight steps and the moments (float16), 3: 40.4, 5: 38.7, 7: 36.1, 9: 37.1,
-// 11: 35.2 ms.
+// eight steps and the moments (float16), 3: 41.1, 5: 38.9, 7: 36.8, 9: 35.8,
+// 11: 35.3 ms.
 #include "static_unit.cuh"
 
 namespace lbrt {

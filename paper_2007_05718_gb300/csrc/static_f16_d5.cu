@@ -2,7 +2,7 @@
 // its launch shared with the 162-direction set.  Two planes a batch; one plane
 // with the flux terms, on a 2D grid and in the alternative batched kernel
 // (static_zc).  Directions streamed ahead of the collision scalars, 128^3 x 42
-// sphere, float16, 40 steps: 2: 7.50, 3: 7.58, 4: 7.92 ms.
+// sphere, float16, 40 steps: 2: 7.36, 3: 7.44, 4: 8.04 ms.
 #include "static_unit.cuh"
 
 namespace lbrt {

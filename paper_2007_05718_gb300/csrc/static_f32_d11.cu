@@ -1,6 +1,6 @@
 // float32 storage, 11 directions per warp (the 162-direction icosahedral set).
 // The directions streamed ahead of the collision scalars (7 of 11) measured at
-// 256^3 x 162, eight steps and the moments: 3: 44.6, 5: 41.8, 7: 39.9, 9: 45.3 ms.
+// 256^3 x 162, eight steps and the moments: 3: 44.1, 5: 41.4, 7: 39.6, 9: 44.9 ms.
 #include "static_unit.cuh"
 
 namespace lbrt {

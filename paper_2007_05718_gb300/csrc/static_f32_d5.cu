@@ -2,7 +2,13 @@
 // and its launch shared with the 162-direction set.  Two planes a batch; one
 // plane with the flux terms, on a 2D grid and in the alternative batched kernel
 // (static_zc).  Directions streamed ahead of the collision scalars, 128^3 x 42
-// sphere, 40 steps: 2: 6.56, 4: 6.22, 5: 6.19 ms.
+// sphere, 40 steps: 2: 6.55, 4: 6.21, 5: 6.18 ms.
+//
+// The flux kernel takes 72 registers, three CTAs of nine warps an SM: its batches
+// wait for one another's chain more than for anything else.  us a step with
+// kappa_1, 64^3 / 128^3 x 42 / 256^3 x 42: two CTAs of 96 registers 64 / 266 /
+// 1719, two planes a batch 62 / 329 / 2136; 72 registers with no direction
+// streamed ahead 48 / 238 / 1570, two of them 46 / 228 / 1511.
 #include "static_unit.cuh"
 
 namespace lbrt {

@@ -38,8 +38,8 @@ int static_plan_lists(int storage, const TilePlan* lists[2], int counts[2]) {
 // Planes per batch of the plan's kernel.  5 directions per warp work two
 // planes a batch, which halves the per-batch work of a warp (128^3 x 42
 // sphere, float16: 0.228 -> 0.175 ms a step).  The flux terms leave no
-// registers for that (64^3 x 42 with kappa_1: two planes took 1.4 times the
-// time of the kernel before, one plane 0.95), and a 2D grid has one plane.
+// registers for that (128^3 x 42 float32 with kappa_1: two planes 308 to 329 us a
+// step, one plane 228), and a 2D grid has one plane.
 int static_zc(int dpt, const Grid& g) { return dpt == 5 && g.dims == 3 && g.nz >= 2 ? 2 : 1; }
 int static_flux_zc(int) { return 1; }
 
