@@ -40,7 +40,7 @@
 //
 // Flux.  With lambda == 0 (no kappa_1 scattering) the collision does not
 // depend on the flux: c1 = dt kappa_0 lambda F = 0.  FLUX == false leaves out
-// the flux partials and the n . c1 terms (they are exact zeros), about a third
+// the flux partials and the n . c1 terms (exact zeros, see unit()), about a third
 // of the packed arithmetic and most of the direction constants.
 //
 // What bounds it.  float32, 256 x 256 x 64 periodic, 162 directions: 1.24 ms,
@@ -491,9 +491,10 @@ __device__ __forceinline__ void static_body(const CUtensorMap& tmap1, const CUte
         Fz += p[192];
       }
     }
+    // lambda == 0: c1 = 0 x F, which is an exact zero, or the NaN of an infinite
+    // opacity or of an infinite F, that is of an infinite E; c0 then takes it
+    if constexpr (!FLUX) Fx = 0.f * E;
     Coef cc = collide_scalars(D.collision, D.lambda_iters, D.dt, inv_d, ka, k0, lam, eta, E, Fx, Fy, Fz);
-    // lambda == 0: c1 = 0 x F, which is an exact zero (or the NaN of an
-    // infinite opacity, which c0 then takes)
     if constexpr (!FLUX) cc.c0 += cc.c1x;
     float* o = coef + ((size_t)(qb & 1) * ZC + j) * NC * 64 + fx;
     float Eh = 0.f;
